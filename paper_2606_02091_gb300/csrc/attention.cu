@@ -18,8 +18,8 @@
 // x 16 rows); one thread streams 64-key K/V tiles by TMA into two 128-byte-swizzled stages;
 // S = Q K^T and O += P V on mma.sync m16n8k16 with bf16 operands and fp32 accumulators, P kept in
 // registers; two to four CTAs fit on an SM.
-// fp32 path: a CUDA-core version of the split with partials in global memory and a second
-// (combine) launch; exact fp32 products.
+// fp32 path: a CUDA-core version (exact fp32 products), with several splits the partials in global
+// memory and a second (combine) launch.
 #include <cuda_fp16.h>
 #include <math.h>
 
@@ -45,8 +45,8 @@ struct AttnArgs {
     const void* kc;       // this layer's cache [max_batch][H_kv][max_ctx][hd]
     const void* vc;
     const int32_t* ctx_len;
-    float* part_o;        // [batch][H_kv][q_tiles][splits][64][hd]
-    float* part_ml;       // [batch][H_kv][q_tiles][splits][64][2]
+    float* part_o;        // fp32 path: [batch][H_kv][q_tiles][splits][16][hd]
+    float* part_ml;       // [batch][H_kv][q_tiles][splits][16][2]
     uint32_t* err;        // device error word (a tile wait that timed out)
     int block_rows;       // rows of one K^d / V^d tensor-map box (min(64, max_batch * B))
     int B, G, hkv, d_q, d_kv, max_ctx, splits, q_tiles;
@@ -1232,84 +1232,182 @@ __global__ void __launch_bounds__(kTThreads, 1) attn_tc_kernel(const __grid_cons
     }
 }
 
-// ------------------------------------------------------------------ CUDA-core path
+// ------------------------------------------------------------------ CUDA-core path (fp32)
+//
+// One CTA per (key split, KV head, 16-row query tile, sequence): 64-key tiles of K and V stream into
+// two shared-memory stages by cp.async; the half-warp of a query row forms four of its tile's
+// scores per lane, keeps the row's online softmax (maximum and sum by shuffles) and then four (or
+// eight) head dims of O per lane, so a row never leaves its warp and a tile costs two CTA barriers.
+// A single split writes the result itself; otherwise the partials go through global memory to a
+// combine launch. Bound by latency at the sizes fp32 drafters have. The earlier form (a warp per
+// query row, one key at a time with a five-shuffle sum each) took 99 us at 16 rows and 136 keys.
 
-template <class T, int HD>
-__global__ void __launch_bounds__(128) attn_simt_kernel(const AttnArgs a) {
+constexpr int kFQ = 16;            // query rows per CTA
+constexpr int kFThreads = 256;
+template <int HD>
+struct F32Attn {
+    static constexpr int KLD = HD + 4;                       // padded K row (floats): no bank conflicts
+    static constexpr int STAGE = kKT * KLD + kKT * HD;       // K then V of one tile
+    static constexpr size_t BYTES = (size_t)(2 * STAGE + kFQ * HD + kFQ * kKT) * sizeof(float);
+};
+
+template <int HD>
+__global__ void __launch_bounds__(kFThreads) attn_simt_kernel(const AttnArgs a, float* __restrict__ out) {
+    using LY = F32Attn<HD>;
+    extern __shared__ __align__(16) float fsm[];
+    float* const Qs = fsm + 2 * LY::STAGE;    // [16][HD]
+    float* const Ps = Qs + kFQ * HD;          // [16][64]
+    const int s = blockIdx.x, g = blockIdx.y % a.hkv, qt = blockIdx.y / a.hkv, b = blockIdx.z;
+    const int tid = threadIdx.x, row = tid >> 4, l16 = tid & 15;
+    const int R = a.B * a.G, rr = qt * kFQ + row;
     pdl_trigger();
     pdl_wait();
-    constexpr int PER = HD / 32;
-    const int s = blockIdx.x, g = blockIdx.y % a.hkv, qt = blockIdx.y / a.hkv, b = blockIdx.z;
-    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-    const int R = a.B * a.G;
     int j_begin, j_end, L;
     key_range(a, b, s, j_begin, j_end, L);
-    const size_t pidx = part_index(a, b, g, qt, s);
-    float* po = a.part_o + pidx * kQT * HD;
-    float* pml = a.part_ml + pidx * kQT * 2;
-    const T* q = static_cast<const T*>(a.q);
-    const T* kd = static_cast<const T*>(a.kd);
-    const T* vd = static_cast<const T*>(a.vd);
-    const T* kc = static_cast<const T*>(a.kc) + ((size_t)b * a.hkv + g) * a.max_ctx * HD;
-    const T* vc = static_cast<const T*>(a.vc) + ((size_t)b * a.hkv + g) * a.max_ctx * HD;
-    for (int r = warp; r < kQT; r += 4) {
-        const int rr = qt * kQT + r;
-        float m = -INFINITY, l = 0.f, acc[PER], qv[PER];
+    const float* kd = static_cast<const float*>(a.kd);
+    const float* vd = static_cast<const float*>(a.vd);
+    const float* kc = static_cast<const float*>(a.kc) + ((size_t)b * a.hkv + g) * a.max_ctx * HD;
+    const float* vc = static_cast<const float*>(a.vc) + ((size_t)b * a.hkv + g) * a.max_ctx * HD;
+    auto load_tile = [&](int j0, int st) {
+        float* K = fsm + st * LY::STAGE;
+        float* V = K + kKT * LY::KLD;
+        for (int i = tid; i < kKT * (HD / 4); i += kFThreads) {
+            const int key = i / (HD / 4), c = (i % (HD / 4)) * 4, j = j0 + key;
+            const float *ks = kc, *vs = vc;
+            const bool in = j < j_end;      // past the range: zero-filled (cp.async of 0 bytes)
+            if (in && j < L) {
+                ks = kc + (size_t)j * HD + c;
+                vs = vc + (size_t)j * HD + c;
+            } else if (in) {
+                const size_t o = ((size_t)b * a.B + (j - L)) * a.d_kv + (size_t)g * HD + c;
+                ks = kd + o;
+                vs = vd + o;
+            }
+            cp_async16(smem_addr(K + key * LY::KLD + c), ks, in);
+            cp_async16(smem_addr(V + key * HD + c), vs, in);
+        }
+        cp_commit();
+    };
+    if (j_begin < j_end) load_tile(j_begin, 0);
+    for (int i = tid; i < kFQ * (HD / 4); i += kFThreads) {
+        const int r = i / (HD / 4), c = (i % (HD / 4)) * 4, q = qt * kFQ + r;
+        float4 v = make_float4(0.f, 0.f, 0.f, 0.f);
+        if (q < R)
+            v = *reinterpret_cast<const float4*>(static_cast<const float*>(a.q) + ((size_t)b * a.B + q / a.G) * a.d_q +
+                                                 (size_t)(g * a.G + q % a.G) * HD + c);
+        *reinterpret_cast<float4*>(Qs + r * HD + c) = v;
+    }
+    float m = -INFINITY, l = 0.f;
+    float4 o[HD / 64];
 #pragma unroll
-        for (int e = 0; e < PER; ++e) acc[e] = 0.f;
-        if (rr < R && j_begin < j_end) {
-            const int kpos = rr / a.G, hh = rr % a.G;
-            const T* qrow = q + ((size_t)b * a.B + kpos) * a.d_q + (size_t)(g * a.G + hh) * HD;
+    for (int e = 0; e < HD / 64; ++e) o[e] = make_float4(0.f, 0.f, 0.f, 0.f);
+    for (int j0 = j_begin, st = 0; j0 < j_end; j0 += kKT, st ^= 1) {
+        if (j0 + kKT < j_end) {
+            load_tile(j0 + kKT, st ^ 1);
+            cp_wait<1>();
+        } else {
+            cp_wait<0>();
+        }
+        __syncthreads();
+        const float* K = fsm + st * LY::STAGE;
+        const float* V = K + kKT * LY::KLD;
+        // scores of keys l16, l16 + 16, + 32, + 48 (four partial sums each)
+        float4 d[4];
 #pragma unroll
-            for (int e = 0; e < PER; ++e) qv[e] = to_f(qrow[lane + 32 * e]);
-            for (int j = j_begin; j < j_end; ++j) {
-                const T *kr, *vr;
-                if (j < L) {
-                    kr = kc + (size_t)j * HD;
-                    vr = vc + (size_t)j * HD;
-                } else {
-                    kr = kd + ((size_t)b * a.B + (j - L)) * a.d_kv + (size_t)g * HD;
-                    vr = vd + ((size_t)b * a.B + (j - L)) * a.d_kv + (size_t)g * HD;
-                }
-                float dot = 0.f;
+        for (int e = 0; e < 4; ++e) d[e] = make_float4(0.f, 0.f, 0.f, 0.f);
+#pragma unroll 4
+        for (int c = 0; c < HD; c += 4) {
+            const float4 q = *reinterpret_cast<const float4*>(Qs + row * HD + c);
 #pragma unroll
-                for (int e = 0; e < PER; ++e) dot = fmaf(qv[e], to_f(kr[lane + 32 * e]), dot);
-                const float sc = warp_sum(dot) * a.scale_log2;
-                const float mn = fmaxf(m, sc);
-                const float corr = exp2f(m - mn), p = exp2f(sc - mn);
-                l = l * corr + p;
-#pragma unroll
-                for (int e = 0; e < PER; ++e) acc[e] = fmaf(p, to_f(vr[lane + 32 * e]), acc[e] * corr);
-                m = mn;
+            for (int e = 0; e < 4; ++e) {
+                const float4 k = *reinterpret_cast<const float4*>(K + (l16 + 16 * e) * LY::KLD + c);
+                d[e].x = fmaf(q.x, k.x, d[e].x);
+                d[e].y = fmaf(q.y, k.y, d[e].y);
+                d[e].z = fmaf(q.z, k.z, d[e].z);
+                d[e].w = fmaf(q.w, k.w, d[e].w);
             }
         }
+        float sc[4], mx = -INFINITY;
 #pragma unroll
-        for (int e = 0; e < PER; ++e) po[(size_t)r * HD + lane + 32 * e] = acc[e];
-        if (lane == 0) {
-            pml[2 * r] = m;
-            pml[2 * r + 1] = l;
+        for (int e = 0; e < 4; ++e) {
+            sc[e] = j0 + l16 + 16 * e < j_end ? ((d[e].x + d[e].y) + (d[e].z + d[e].w)) * a.scale_log2 : -INFINITY;
+            mx = fmaxf(mx, sc[e]);
         }
+#pragma unroll
+        for (int w = 8; w > 0; w >>= 1) mx = fmaxf(mx, __shfl_xor_sync(0xffffffffu, mx, w));
+        const float mn = fmaxf(m, mx), corr = exp2f(m - mn);
+        float sum = 0.f;
+#pragma unroll
+        for (int e = 0; e < 4; ++e) {
+            const float p = exp2f(sc[e] - mn);
+            Ps[row * kKT + l16 + 16 * e] = p;
+            sum += p;
+        }
+#pragma unroll
+        for (int w = 8; w > 0; w >>= 1) sum += __shfl_xor_sync(0xffffffffu, sum, w);
+        l = l * corr + sum;
+        m = mn;
+        __syncwarp();
+        // O[row][4 l16 .. + 3] (and + 64 at head_dim 128) over the tile's keys
+#pragma unroll
+        for (int e = 0; e < HD / 64; ++e) {
+            o[e].x *= corr;
+            o[e].y *= corr;
+            o[e].z *= corr;
+            o[e].w *= corr;
+        }
+#pragma unroll 4
+        for (int j = 0; j < kKT; j += 4) {
+            const float4 p4 = *reinterpret_cast<const float4*>(Ps + row * kKT + j);
+            const float p[4] = {p4.x, p4.y, p4.z, p4.w};
+#pragma unroll
+            for (int u = 0; u < 4; ++u)
+#pragma unroll
+                for (int e = 0; e < HD / 64; ++e) {
+                    const float4 v = *reinterpret_cast<const float4*>(V + (j + u) * HD + 64 * e + 4 * l16);
+                    o[e].x = fmaf(p[u], v.x, o[e].x);
+                    o[e].y = fmaf(p[u], v.y, o[e].y);
+                    o[e].z = fmaf(p[u], v.z, o[e].z);
+                    o[e].w = fmaf(p[u], v.w, o[e].w);
+                }
+        }
+        __syncthreads();   // the stage and P are free for the next tile
+    }
+    if (a.splits == 1) {
+        if (rr >= R) return;
+        float* dst = out + ((size_t)b * a.B + rr / a.G) * a.d_q + (size_t)(g * a.G + rr % a.G) * HD + 4 * l16;
+#pragma unroll
+        for (int e = 0; e < HD / 64; ++e)
+            *reinterpret_cast<float4*>(dst + 64 * e) = make_float4(o[e].x / l, o[e].y / l, o[e].z / l, o[e].w / l);
+        return;
+    }
+    const size_t pr = part_index(a, b, g, qt, s) * kFQ + row;
+#pragma unroll
+    for (int e = 0; e < HD / 64; ++e) *reinterpret_cast<float4*>(a.part_o + pr * HD + 64 * e + 4 * l16) = o[e];
+    if (l16 == 0) {
+        a.part_ml[2 * pr] = m;
+        a.part_ml[2 * pr + 1] = l;
     }
 }
 
 // ------------------------------------------------------------------ combine
 
-template <class T, int HD>
-__global__ void attn_combine_kernel(const AttnArgs a, T* __restrict__ out) {
+template <int HD>
+__global__ void attn_combine_kernel(const AttnArgs a, float* __restrict__ out) {
     pdl_trigger();
     pdl_wait();
     const int rr = blockIdx.x, g = blockIdx.y, b = blockIdx.z;
-    const int qt = rr / kQT, r = rr % kQT;
+    const int qt = rr / kFQ, r = rr % kFQ;
     const int kpos = rr / a.G, hh = rr % a.G;
     float M = -INFINITY;
     for (int s = 0; s < a.splits; ++s)
-        M = fmaxf(M, a.part_ml[(part_index(a, b, g, qt, s) * kQT + r) * 2]);
-    float den = 0.f, num[HD / 64 > 0 ? HD / 64 : 1];
+        M = fmaxf(M, a.part_ml[(part_index(a, b, g, qt, s) * kFQ + r) * 2]);
     constexpr int PER = HD / 64;
+    float den = 0.f, num[PER];
 #pragma unroll
     for (int e = 0; e < PER; ++e) num[e] = 0.f;
     for (int s = 0; s < a.splits; ++s) {
-        const size_t pi = part_index(a, b, g, qt, s) * kQT + r;
+        const size_t pi = part_index(a, b, g, qt, s) * kFQ + r;
         const float ms = a.part_ml[pi * 2];
         if (ms == -INFINITY) continue;
         const float w = exp2f(ms - M);
@@ -1317,9 +1415,9 @@ __global__ void attn_combine_kernel(const AttnArgs a, T* __restrict__ out) {
 #pragma unroll
         for (int e = 0; e < PER; ++e) num[e] = fmaf(w, a.part_o[pi * HD + threadIdx.x + 64 * e], num[e]);
     }
-    T* orow = out + ((size_t)b * a.B + kpos) * a.d_q + (size_t)(g * a.G + hh) * HD;
+    float* orow = out + ((size_t)b * a.B + kpos) * a.d_q + (size_t)(g * a.G + hh) * HD;
 #pragma unroll
-    for (int e = 0; e < PER; ++e) orow[threadIdx.x + 64 * e] = from_f<T>(num[e] / den);
+    for (int e = 0; e < PER; ++e) orow[threadIdx.x + 64 * e] = num[e] / den;
 }
 
 template <int HD>
@@ -1445,30 +1543,42 @@ int tc_active_clusters(int sp) {
     return n;
 }
 
-template <class T, int HD>
+template <int HD>
 cudaError_t run_simt(dflare_ctx* c, const AttnArgs& a, cudaStream_t s) {
-    cudaError_t e = launch_kernel(c->pdl, attn_simt_kernel<T, HD>,
-                                  dim3(a.splits, a.hkv * a.q_tiles, c->batch), dim3(128), 0, s, a);
+    static PerDeviceOnce configured;
+    cudaError_t e = configured([] {
+        return cudaFuncSetAttribute(attn_simt_kernel<HD>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                    (int)F32Attn<HD>::BYTES);
+    });
     if (e != cudaSuccess) return e;
-    return launch_kernel(c->pdl, attn_combine_kernel<T, HD>, dim3(a.B * a.G, a.hkv, c->batch),
-                         dim3(64), 0, s, a, static_cast<T*>(c->attn));
+    e = launch_kernel(c->pdl, attn_simt_kernel<HD>, dim3(a.splits, a.hkv * a.q_tiles, c->batch), dim3(kFThreads),
+                      F32Attn<HD>::BYTES, s, a, static_cast<float*>(c->attn));
+    if (e != cudaSuccess || a.splits == 1) return e;
+    return launch_kernel(c->pdl, attn_combine_kernel<HD>, dim3(a.B * a.G, a.hkv, c->batch),
+                         dim3(64), 0, s, a, static_cast<float*>(c->attn));
 }
 
 }  // namespace
 
-// CUDA-core (fp32) path: enough splits for about two CTAs per SM over batch x H_kv x q_tiles,
-// none shorter than 256 keys at the host's upper bound of the context length; partials go
-// through global memory to a combine launch. The device derives the actual ranges from the true
-// lengths, so a stale bound (e.g. a replayed graph) only costs speed.
+static int attention_q_tiles_f32(const dflare_config& g) {
+    return (g.block * (g.n_q_heads / g.n_kv_heads) + kFQ - 1) / kFQ;
+}
+
+// CUDA-core (fp32) path: one split up to three 64-key tiles (a tile costs about 1.5 us, the partials
+// and the combine launch about 3), else one per two tiles, as many as fit two CTAs per SM. The device
+// derives the actual ranges from the true lengths, so a stale bound (e.g. a replayed graph) only
+// costs speed.
 int attention_splits(const dflare_config& g, int batch, int num_sms, int len_ub) {
-    const int G = g.n_q_heads / g.n_kv_heads;
-    const int q_tiles = (g.block * G + kQT - 1) / kQT;
+    const int q_tiles = attention_q_tiles_f32(g);
     const int base = batch * g.n_kv_heads * q_tiles;
-    // CUDA-core path: each warp walks its query rows over the split's keys one key at a time, so
-    // splits of at least 64 keys, as many as give two CTAs per SM
-    int sp = (2 * num_sms + base - 1) / base;
-    sp = std::min(sp, (len_ub + g.block + 63) / 64);
-    return std::max(1, sp);
+    const int tiles = (len_ub + g.block + kKT - 1) / kKT;
+    if (tiles <= 3) return 1;
+    return std::max(1, std::min((2 * num_sms + base - 1) / base, (tiles + 1) / 2));
+}
+
+// rows of the partial buffers of a batch (the split count grows with the context bound)
+size_t attention_partial_rows_f32(const dflare_config& g, int batch, int num_sms) {
+    return (size_t)batch * g.n_kv_heads * attention_q_tiles_f32(g) * attention_splits(g, batch, num_sms, g.max_ctx) * kFQ;
 }
 
 // Tensor-core path: the splits of one (sequence, head, query tile) are one cluster of 1, 2, 4, 8
@@ -1571,8 +1681,9 @@ cudaError_t launch_attention(dflare_ctx* c, int layer, cudaStream_t s) {
     a.q_tiles = (a.B * a.G + kQT - 1) / kQT;
     a.scale_log2 = 1.4426950408889634f / sqrtf((float)g.head_dim);
     if (g.dtype == DFLARE_F32) {
+        a.q_tiles = attention_q_tiles_f32(g);
         a.splits = attention_splits(g, c->batch, c->num_sms, c->ctx_ub);
-        return g.head_dim == 64 ? run_simt<float, 64>(c, a, s) : run_simt<float, 128>(c, a, s);
+        return g.head_dim == 64 ? run_simt<64>(c, a, s) : run_simt<128>(c, a, s);
     }
     a.err = c->err;
     if (c->qkv32 && !(g.flags & (DFLARE_FLAG_DETERMINISTIC | DFLARE_FLAG_SIMT_GEMM))) {

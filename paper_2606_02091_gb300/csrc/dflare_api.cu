@@ -15,7 +15,7 @@
 using namespace dfl;
 
 namespace dfl {
-int attention_splits(const dflare_config& g, int batch, int num_sms, int len_ub);
+size_t attention_partial_rows_f32(const dflare_config& g, int batch, int num_sms);
 }
 
 namespace {
@@ -351,13 +351,9 @@ dflare_status dflare_create(const dflare_config* cfg, dflare_ctx** out) {
     const size_t rows = (size_t)g.max_batch * B, mrows = (size_t)g.max_batch * (B > 1 ? B - 1 : 1);
     const size_t kv = D * g.max_batch * d_kv * (size_t)g.max_ctx;
     // split-KV partial buffers sized for the largest batch x splits product
-    const int G = g.n_q_heads / g.n_kv_heads;
-    const int q_tiles = (g.block * G + 63) / 64;
     size_t part_rows = 1;   // split-KV partials in global memory: the fp32 path only
-    for (int b = 1; b <= g.max_batch && g.dtype == DFLARE_F32; ++b) {
-        const size_t r = (size_t)b * g.n_kv_heads * q_tiles * attention_splits(g, b, c->num_sms, g.max_ctx) * 64;
-        if (r > part_rows) part_rows = r;
-    }
+    for (int b = 1; b <= g.max_batch && g.dtype == DFLARE_F32; ++b)
+        part_rows = std::max(part_rows, attention_partial_rows_f32(g, b, c->num_sms));
     c->ws_floats = (size_t)8 << 20;
     c->tile_cnt_n = 8192;
 #define ALLOC(ptr, bytes)                                                                    \

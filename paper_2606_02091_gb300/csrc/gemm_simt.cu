@@ -1,94 +1,146 @@
 // CUDA-core projection GEMM: the fp32 storage mode's GEMM (exact fp32 products, which the
 // tensor cores do not offer) and, for bf16, a diagnostic cross-check of the tcgen05 GEMM.
-// One CTA computes 128 output features x 16 tokens (x2 accumulators for SwiGLU) over the whole
-// K range, then hands the tile to the shared epilogue.
+//
+// The fp32 drafters are small (hidden size of a few hundred, a handful of token rows), so a
+// projection is bound by the latency of its longest chain, not by bandwidth. One CTA takes 32
+// weight rows x TT tokens over the whole K range, one warp four rows: a lane holds 4 consecutive k
+// of every 128, multiplies them with the same k of all TT tokens (64 sums in registers at 16
+// tokens), and the 32 lanes' sums are added in a butterfly that halves the values a lane holds at
+// each step. No shared memory and no barrier until the epilogue, the first weights are loaded
+// before the dependency wait, and a lane's serial chain is K / 32 FMAs per sum. Each 16-byte load
+// feeds 16 (weights: 4 TT) FMAs, so the same form also runs a fill of hundreds of tokens near the
+// L1 limit. The earlier form (128 rows x 16 tokens per CTA, K in shared-memory chunks of 16 between
+// two barriers) waited a memory round trip per chunk (ncu: 32 us at K 256, 92 us at K 768). With this
+// kernel and the fp32 attention of attention.cu the first step of a 128-position sequence on the fp32
+// drafter (d 256, 4 layers, block 8) went from 968 to 153 us.
 #include "epilogue.cuh"
 
 namespace dfl {
 namespace {
 
-constexpr int kTN = 128;   // features per CTA
-constexpr int kTT = 16;    // tokens per CTA
-constexpr int kTK = 16;    // K chunk
+constexpr int kRows = 32;      // weight rows per CTA: two groups of 16 features (SwiGLU: one group
+                               // of gate and the same 16 features of up)
+constexpr int kSimtThreads = 256;
 
-template <class T>
-__global__ void __launch_bounds__(256) gemm_simt_kernel(const T* __restrict__ A, const T* __restrict__ A2,
-                                                        const T* __restrict__ Bm, int n, int k,
-                                                        int m_tok, long long a_group_rows,
-                                                        long long b_group_rows, int b_shared,
-                                                        int b_kgroup, int n_tiles, EpiParams ep) {
+__device__ __forceinline__ float4 ld4(const float* p) { return *reinterpret_cast<const float4*>(p); }
+__device__ __forceinline__ float4 ld4(const bf16* p) {
+    const uint2 u = *reinterpret_cast<const uint2*>(p);
+    return make_float4(__uint_as_float(u.x << 16), __uint_as_float(u.x & 0xFFFF0000u),
+                       __uint_as_float(u.y << 16), __uint_as_float(u.y & 0xFFFF0000u));
+}
+
+// TT: tokens per CTA (8 or 16). blockIdx.x = group * n_slices + slice, blockIdx.y = token chunk.
+template <class T, int TT>
+__global__ void __launch_bounds__(kSimtThreads) gemm_simt_kernel(
+    const T* __restrict__ A, const T* __restrict__ A2, const T* __restrict__ Bm, int n, int k, int m_tok,
+    long long a_group_rows, long long b_group_rows, int b_shared, int b_kgroup, int n_slices, EpiParams ep) {
+    __shared__ __align__(16) float tile[2 * kEpiChunk * 128];   // the epilogue's [acc][token][feature]
+    const int slice = blockIdx.x % n_slices, group = blockIdx.x / n_slices;
+    const int tok0 = blockIdx.y * TT;
+    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+    // the CTA's two groups of 16 features; a projection with a rotary epilogue takes a group and its
+    // rotary partner half a head further, so that the epilogue finds both in its tile
+    int f_a, f_b;
+    if (A2) {
+        f_a = f_b = slice * 16;
+    } else if (ep.kind == EPI_QKV || ep.kind == EPI_KV_APPEND) {
+        const int q = slice & 3;
+        f_a = (slice >> 2) * 128 + (ep.head_dim == 64 ? (q >> 1) * 64 + (q & 1) * 16 : q * 16);
+        f_b = f_a + (ep.head_dim >> 1);
+    } else {
+        f_a = slice * 32;
+        f_b = f_a + 16;
+    }
+    const int sub = (warp & 3) * 4;                     // the warp's first row within its group
+    const int row0 = (warp < 4 ? f_a : f_b) + sub;
+    const T* Ag = (A2 && warp >= 4 ? A2 : A) + (size_t)group * a_group_rows * k;
+    const T* wp[4];
+#pragma unroll
+    for (int f = 0; f < 4; ++f) wp[f] = Ag + (size_t)min(row0 + f, n - 1) * k + 4 * lane;   // rows past n: not stored
+    const float4 zero = make_float4(0.f, 0.f, 0.f, 0.f);
+    float4 w[4];
+#pragma unroll
+    for (int f = 0; f < 4; ++f) w[f] = 4 * lane < k ? ld4(wp[f]) : zero;
     pdl_wait();
     pdl_trigger();   // after the wait: see gemm_tc_kernel
-    __shared__ float sA[2][kTN][kTK + 1];
-    __shared__ float sB[kTT][kTK + 1];
-    __shared__ __align__(16) float tile[2 * kTT * kTN];
-    const int n_tile = blockIdx.x % n_tiles, group = blockIdx.x / n_tiles;
-    const int tok0 = blockIdx.y * kTT;
-    const int na = A2 ? 2 : 1;
-    const int tid = threadIdx.x;
-    const int f = tid & 127, tg = tid >> 7;   // feature f, tokens tg*8 .. tg*8+7
-    const T* Ag = A + (size_t)group * a_group_rows * k;
-    const T* A2g = A2 ? A2 + (size_t)group * a_group_rows * k : nullptr;
-    const T* Bg = Bm + (size_t)(b_shared ? 0 : group) * b_group_rows * k;
-    float acc[2][8];
+    const T* Bg = Bm + (size_t)(b_shared || b_kgroup > 0 ? 0 : group) * b_group_rows * k;
+    const size_t b_ld = b_kgroup > 0 ? b_kgroup : k;    // elements between token rows
+    float acc[4 * TT];
 #pragma unroll
-    for (int a = 0; a < 2; ++a)
-#pragma unroll
-        for (int i = 0; i < 8; ++i) acc[a][i] = 0.f;
-    for (int k0 = 0; k0 < k; k0 += kTK) {
-        __syncthreads();
-        for (int idx = tid; idx < kTN * kTK; idx += 256) {
-            const int r = idx / kTK, cc = idx % kTK;
-            const int row = n_tile * kTN + r, col = k0 + cc;
-            const bool in = row < n && col < k;
-            sA[0][r][cc] = in ? to_f(Ag[(size_t)row * k + col]) : 0.f;
-            if (na == 2) sA[1][r][cc] = in ? to_f(A2g[(size_t)row * k + col]) : 0.f;
+    for (int i = 0; i < 4 * TT; ++i) acc[i] = 0.f;
+    for (int c0 = 0; c0 < k; c0 += 128) {
+        const int col = c0 + 4 * lane;
+        const bool in = col < k;
+        const T* bp = Bg + col;
+        if (b_kgroup > 0) {   // contraction over stacked activation groups (Eq. 1)
+            const int z = col / b_kgroup;
+            bp = Bm + (size_t)z * b_group_rows * b_kgroup + (col - z * b_kgroup);
         }
-        for (int idx = tid; idx < kTT * kTK; idx += 256) {
-            const int r = idx / kTK, cc = idx % kTK;
-            const int tok = tok0 + r, col = k0 + cc;
-            float v = 0.f;
-            if (tok < m_tok && col < k) {
-                if (b_kgroup > 0) {   // contraction over stacked activation groups (Eq. 1)
-                    const int z = col / b_kgroup;
-                    v = to_f(Bm[((size_t)z * b_group_rows + tok) * b_kgroup + (col - z * b_kgroup)]);
-                } else {
-                    v = to_f(Bg[(size_t)tok * k + col]);
-                }
-            }
-            sB[r][cc] = v;
-        }
-        __syncthreads();
-        for (int a = 0; a < na; ++a)
-#pragma unroll 4
-            for (int cc = 0; cc < kTK; ++cc) {
-                const float w = sA[a][f][cc];
+        float4 x[TT];
 #pragma unroll
-                for (int i = 0; i < 8; ++i) acc[a][i] = fmaf(w, sB[tg * 8 + i][cc], acc[a][i]);
+        for (int t = 0; t < TT; ++t) x[t] = in ? ld4(bp + (size_t)min(tok0 + t, m_tok - 1) * b_ld) : zero;
+        float4 wn[4];
+        const bool more = col + 128 < k;
+#pragma unroll
+        for (int f = 0; f < 4; ++f) wn[f] = more ? ld4(wp[f] + c0 + 128) : zero;
+#pragma unroll
+        for (int f = 0; f < 4; ++f)
+#pragma unroll
+            for (int t = 0; t < TT; ++t) {
+                float a = acc[f * TT + t];
+                a = fmaf(w[f].x, x[t].x, a);
+                a = fmaf(w[f].y, x[t].y, a);
+                a = fmaf(w[f].z, x[t].z, a);
+                acc[f * TT + t] = fmaf(w[f].w, x[t].w, a);
             }
+#pragma unroll
+        for (int f = 0; f < 4; ++f) w[f] = wn[f];
     }
-    for (int a = 0; a < na; ++a)
+    // add the 32 lanes' sums: at each step a lane keeps one half of its values (the upper half when
+    // its lane bit is set) and gives the other away; afterwards it holds values 4 TT / 32 * lane ..
+    constexpr int kLeft = 4 * TT / 32;
 #pragma unroll
-        for (int i = 0; i < 8; ++i) tile[(a * kTT + tg * 8 + i) * kTN + f] = acc[a][i];
+    for (int o = 16, half = 2 * TT; o > 0; o >>= 1, half >>= 1) {
+        const bool up = lane & o;
+#pragma unroll
+        for (int i = 0; i < half; ++i) {
+            const float give = up ? acc[i] : acc[i + half];
+            const float keep = up ? acc[i + half] : acc[i];
+            acc[i] = keep + __shfl_xor_sync(0xffffffffu, give, o);
+        }
+    }
+    float* const dst = tile + (A2 && warp >= 4 ? kEpiChunk * 128 : 0) + (row0 & 127);
+#pragma unroll
+    for (int i = 0; i < kLeft; ++i) {
+        const int v = lane * kLeft + i;                 // value f * TT + t
+        dst[(v % TT) * 128 + v / TT] = acc[i];
+    }
     __syncthreads();
-    if (tid < 128) apply_epilogue<T>(ep, tile, group, n_tile, tok0, tid);
+    const int c = threadIdx.x >> 1, g = threadIdx.x & 1;
+    if (c < TT && !(A2 && g)) {
+        const int f0 = g ? f_b : f_a;
+        apply_epilogue<T>(ep, tile, group, f0 >> 7, tok0, c * 8 + ((f0 & 127) >> 4));
+    }
+}
+
+template <class T>
+cudaError_t launch_t(dflare_ctx* c, const GemmDesc& g, cudaStream_t s) {
+    const int per = g.a2 ? 16 : kRows;
+    const int n_slices = (g.n + per - 1) / per;
+    const long long a_gr = g.a_group_rows > 0 ? g.a_group_rows : g.n;
+    const int tt = g.m_tok <= 8 ? 8 : 16;
+    return launch_kernel(c->pdl, tt == 8 ? gemm_simt_kernel<T, 8> : gemm_simt_kernel<T, 16>,
+                         dim3(n_slices * g.groups, (g.m_tok + tt - 1) / tt), dim3(kSimtThreads), 0, s,
+                         (const T*)g.a, (const T*)g.a2, (const T*)g.b, g.n, g.k, g.m_tok, a_gr, g.b_group_rows,
+                         g.b_shared, g.b_kgroup, n_slices, g.ep);
 }
 
 }  // namespace
 
 cudaError_t launch_gemm_simt(dflare_ctx* c, const GemmDesc& g, cudaStream_t s) {
     if (g.m_tok <= 0 || g.n <= 0) return cudaSuccess;
-    const int n_tiles = (g.n + kTN - 1) / kTN;
     if (g.b_kgroup > 0 && (g.k % g.b_kgroup != 0 || g.groups != 1)) return cudaErrorInvalidValue;
-    dim3 grid(n_tiles * g.groups, (g.m_tok + kTT - 1) / kTT);
-    const long long a_gr = g.a_group_rows > 0 ? g.a_group_rows : g.n;
-    if (c->cfg.dtype == DFLARE_F32)
-        return launch_kernel(c->pdl, gemm_simt_kernel<float>, grid, dim3(256), 0, s,
-                             (const float*)g.a, (const float*)g.a2, (const float*)g.b, g.n, g.k,
-                             g.m_tok, a_gr, g.b_group_rows, g.b_shared, g.b_kgroup, n_tiles, g.ep);
-    return launch_kernel(c->pdl, gemm_simt_kernel<bf16>, grid, dim3(256), 0, s, (const bf16*)g.a,
-                         (const bf16*)g.a2, (const bf16*)g.b, g.n, g.k, g.m_tok, a_gr,
-                         g.b_group_rows, g.b_shared, g.b_kgroup, n_tiles, g.ep);
+    return c->cfg.dtype == DFLARE_F32 ? launch_t<float>(c, g, s) : launch_t<bf16>(c, g, s);
 }
 
 }  // namespace dfl

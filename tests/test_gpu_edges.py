@@ -1,0 +1,62 @@
+"""Kernels of the draft path at the sizes where their tilings have edges, against the oracle.
+
+The checks and tolerances are those of tests/harness.py (fp32 storage: 1e-5 element by element with the
+floor at the tensor's rms; bf16 storage: 2e-2, see there)."""
+import numpy as np
+import pytest
+
+import synth
+from tests.harness import GpuSide, check_kv, check_rows, check_tokens, f64, oracle_for
+
+pytestmark = pytest.mark.gpu
+
+
+def _shape(**kw):
+    base = dict(d=256, n_draft_layers=2, n_target_layers=2, n_q_heads=4, n_kv_heads=2, head_dim=64, ffn=256,
+                vocab=700, block=8)
+    base.update(kw)
+    return synth.Shape(**base)
+
+
+def _step_matches_oracle(w, flags=0):
+    """A fill of w.ctx_lens in one call, every cached key and value, and one drafted block."""
+    g = GpuSide(w, flags=flags)
+    o = oracle_for(w, g.W)
+    got = f64(g.fuse(w.ctx_lens))
+    for b, n in enumerate(w.ctx_lens):
+        F = o.fuse_context(b, synth.hidden_states(w, b, 0, n))
+        for i in range(w.shape.n_draft_layers):
+            check_rows(w, got[i, b, :n], F[i], f"F seq {b} layer {i}")
+            k, v = g.lib.read_kv(i, b, 0, n)
+            check_kv(w, o, f64(k), f64(v), got[i, b, :n], np.arange(n), i, f"seq {b} layer {i}")
+    x_t = synth.initial_tokens(w)
+    tok, logits, hidden = g.draft(x_t)
+    for b in range(w.batch):
+        ot, ol, oh = o.draft_block(b, int(x_t[b]))
+        for i in range(oh.shape[0]):
+            check_rows(w, hidden[i, b], oh[i], f"seq {b} hidden after layer {i - 1}")
+        check_rows(w, logits[b], ol, f"seq {b} logits")
+        check_tokens(w, o, tok[b], logits[b], hidden[-1, b], ot, ol, f"seq {b}")
+    assert g.lib.device_error() == 0
+
+
+# fp32: 8- and 16-token CTAs (7, 8, 9, 16, 17 and 34 rows), contractions that are no multiple of 128,
+# feature counts that are no multiple of 32 (the vocabulary), one and several key splits, a tile of
+# keys that the context and the block share, more than one 16-row query tile, both head sizes
+F32_CASES = [
+    synth.Workload("f32_b1", _shape(dtype="f32", d=192, ffn=320, vocab=1003, block=8), (56,), 0.8, 31, False),
+    synth.Workload("f32_block9", _shape(dtype="f32", d=320, block=9, vocab=129), (184, 1), 0.8, 32, False),
+    synth.Workload("f32_block17_hd128", _shape(dtype="f32", head_dim=128, n_q_heads=8, block=17, vocab=97), (700, 65), 0.8, 33, False),
+    synth.Workload("f32_block1", _shape(dtype="f32", block=1, n_q_heads=2), (191,), 0.8, 34, False),
+]
+
+
+@pytest.mark.parametrize("w", F32_CASES, ids=lambda w: w.name)
+def test_fp32_kernels_match_oracle(w):
+    _step_matches_oracle(w)
+
+
+def test_simt_gemm_on_bf16_matches_oracle():
+    """The CUDA-core GEMM on bf16 weights (a cross-check of the tensor-core GEMM)."""
+    from paper_2606_02091_gb300 import FLAG_SIMT_GEMM
+    _step_matches_oracle(synth.Workload("simt_bf16", _shape(d=320, ffn=192, vocab=333, block=9), (40, 3), 0.8, 35), FLAG_SIMT_GEMM)
