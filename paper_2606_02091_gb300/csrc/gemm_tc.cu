@@ -735,6 +735,18 @@ cudaError_t launch_gemm_tc(dflare_ctx* c, const GemmDesc& g, cudaStream_t s, std
     TcArgs a;
     memset(&a, 0, sizeof(a));
     a.bn = g.m_tok <= 256 ? ((g.m_tok + 15) / 16) * 16 : 256;
+    // A projection with few weight tiles is divided over the SMs by tokens (tiles of 64 rows at
+    // least) before it is divided along K, where K splits would go through the workspace: at 240
+    // tokens each split writes 120 KB of partials and the last CTA of a tile reads all of them
+    // back, while token tiles only read the weights again from L2. LM head of 4096 entries, d 4096:
+    // one layer with 240 such rows 237.1 -> 224.8 us, with 248 rows and long contexts 373.7 ->
+    // 353.4 us (4 K splits of a 256-token tile against 4 tiles of 64).
+    const bool ws_splits = g.ep.kind != EPI_RED32 && !(g.ep.kind == EPI_RESID && !(c->cfg.flags & DFLARE_FLAG_DETERMINISTIC));
+    const long long w_tiles = (long long)g.groups * ((g.n + kBM - 1) / kBM);
+    // (DFlash's FC keeps K splits: its contraction of T d is long enough to outweigh the partials)
+    while (ws_splits && g.force_splits <= 0 && g.b_kgroup == 0 && a.bn >= 128 &&
+           w_tiles * ((g.m_tok + a.bn / 2 - 1) / (a.bn / 2)) <= c->num_sms)
+        a.bn = (a.bn / 2 + 15) / 16 * 16;
     // With token tiles of 128 or more rows the GEMM is bound by the tensor pipeline, not by HBM:
     // two adjacent 128-row weight tiles can then share one activation tile (two accumulators, as
     // the SwiGLU gate and up tiles do), a third fewer shared-memory bytes per FLOP. At 256 token
