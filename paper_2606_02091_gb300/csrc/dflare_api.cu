@@ -537,12 +537,19 @@ dflare_status draft_block_impl(dflare_ctx* c, const int32_t* last_token, int32_t
     const size_t d_q = (size_t)g.n_q_heads * g.head_dim, d_kv = (size_t)g.n_kv_heads * g.head_dim;
     const int rows = c->batch * g.block;
     const size_t hid_stride = (size_t)c->batch * B * d;
+    // The caller's copies of the residual stream and of the logits are written by the kernels that
+    // read these anyway (the next norm, the argmax or the draw), 16 bytes at a time, so an unaligned
+    // buffer, and the last layer of a block without mask rows, take a copy of their own. As copies
+    // they cost a launch each, cut the dependent launches apart and read everything again.
+    const bool hid_fused = hidden_out && reinterpret_cast<uintptr_t>(hidden_out) % 16 == 0;
+    const bool log_fused = logits_out && reinterpret_cast<uintptr_t>(logits_out) % 16 == 0;
+    auto hid = [&](int i) { return hidden_out + (size_t)i * hid_stride; };
     {
         Trace t(c, "embed", s);
-        CUDA_TRY(launch_embed(c, last_token, s));
+        CUDA_TRY(launch_embed(c, last_token, s, hid_fused ? hid(0) : nullptr));
     }
-    if (hidden_out)
-        CUDA_TRY(cudaMemcpyAsync(hidden_out, c->x, hid_stride * 4, cudaMemcpyDeviceToDevice, s));
+    if (hidden_out && !hid_fused)
+        CUDA_TRY(cudaMemcpyAsync(hid(0), c->x, hid_stride * 4, cudaMemcpyDeviceToDevice, s));
     // bf16 tensor-core path: the Q/K^d/V^d splits add their fp32 partials into qkv32 with L2
     // reductions and the attention applies the rotary embedding and rounds as it loads them (no
     // split-K workspace, tile counter or last-CTA epilogue on the critical path); qkv32 is cleared
@@ -553,7 +560,7 @@ dflare_status draft_block_impl(dflare_ctx* c, const int32_t* last_token, int32_t
         if (i > 0) {
             Trace t(c, "rmsnorm", s);
             CUDA_TRY(launch_rmsnorm(c, at(c->w.attn_norm, i * d, esz), rows, false, c->xn, s,
-                                    red32 ? c->qkv32 : nullptr));
+                                    red32 ? c->qkv32 : nullptr, hid_fused ? hid(i) : nullptr));
         }
         // Q = X~ W_Q, K^d = X~ W_K^d, V^d = X~ W_V^d with the rotary embedding (Eq. 4)
         GemmDesc q{};
@@ -637,16 +644,16 @@ dflare_status draft_block_impl(dflare_ctx* c, const int32_t* last_token, int32_t
         dn.ep.resid = c->x;
         dn.ep.ld_resid = g.d;
         if ((st = traced_gemm(c, "gemm_down", dn, s)) != DFLARE_OK) return st;
-        if (hidden_out)
-            CUDA_TRY(cudaMemcpyAsync(hidden_out + (size_t)(i + 1) * hid_stride, c->x, hid_stride * 4,
-                                     cudaMemcpyDeviceToDevice, s));
+        if (hidden_out && (!hid_fused || (i + 1 == g.n_draft_layers && g.block < 2)))
+            CUDA_TRY(cudaMemcpyAsync(hid(i + 1), c->x, hid_stride * 4, cudaMemcpyDeviceToDevice, s));
     }
     if (g.block < 2) return DFLARE_OK;
     // final RMSNorm of the mask rows, LM head, greedy argmax (Sec. 3.2)
     const int mrows = c->batch * (g.block - 1);
     {
         Trace t(c, "rmsnorm", s);
-        CUDA_TRY(launch_rmsnorm(c, c->w.final_norm, mrows, true, c->xh, s));
+        CUDA_TRY(launch_rmsnorm(c, c->w.final_norm, mrows, true, c->xh, s, nullptr,
+                                hid_fused ? hid(g.n_draft_layers) : nullptr));
     }
     GemmDesc h{};
     h.a = c->w.lm_head;
@@ -666,12 +673,12 @@ dflare_status draft_block_impl(dflare_ctx* c, const int32_t* last_token, int32_t
     if (st != DFLARE_OK) return st;
     if (smp) {
         Trace t(c, "sample", s);
-        CUDA_TRY(launch_sample(c, mrows, smp->inv_t, smp->seed, smp->step, draft_tokens, s));
+        CUDA_TRY(launch_sample(c, mrows, smp->inv_t, smp->seed, smp->step, draft_tokens, s, log_fused ? logits_out : nullptr));
     } else {
         Trace t(c, "argmax", s);
-        CUDA_TRY(launch_argmax(c, c->logits, mrows, draft_tokens, s));
+        CUDA_TRY(launch_argmax(c, c->logits, mrows, draft_tokens, s, log_fused ? logits_out : nullptr));
     }
-    if (logits_out)
+    if (logits_out && !log_fused)
         CUDA_TRY(cudaMemcpyAsync(logits_out, c->logits, (size_t)mrows * g.vocab * 4,
                                  cudaMemcpyDeviceToDevice, s));
     return DFLARE_OK;

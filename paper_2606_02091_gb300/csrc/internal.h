@@ -241,15 +241,18 @@ cudaError_t launch_fusion_alpha(dflare_ctx* c, cudaStream_t s);
 cudaError_t launch_fuse_begin(dflare_ctx* c, const int32_t* n_new, int n_max, cudaStream_t s);
 cudaError_t launch_fuse_layers(dflare_ctx* c, const void* hidden, int n_max, void* fused_out,
                                cudaStream_t s);
-cudaError_t launch_embed(dflare_ctx* c, const int32_t* last_token, cudaStream_t s);
-// zero32 (optional): the fp32 Q/K^d/V^d sums of the next projection, rows x (d_q + 2 d_kv), cleared
+// copy (optional, 16-byte aligned): the block rows of the residual stream, [batch*B][d] fp32
+cudaError_t launch_embed(dflare_ctx* c, const int32_t* last_token, cudaStream_t s, float* copy = nullptr);
+// zero32 (optional): the fp32 Q/K^d/V^d sums of the next projection, rows x (d_q + 2 d_kv), cleared;
+// copy as above
 cudaError_t launch_rmsnorm(dflare_ctx* c, const void* gain, int rows, bool gather_mask_rows,
-                           void* out, cudaStream_t s, float* zero32 = nullptr);
+                           void* out, cudaStream_t s, float* zero32 = nullptr, float* copy = nullptr);
 cudaError_t launch_attention(dflare_ctx* c, int layer, cudaStream_t s);
+// copy (optional, 16-byte aligned): receives the logits, [rows][V]
 cudaError_t launch_argmax(dflare_ctx* c, const float* logits, int rows, int32_t* tokens,
-                          cudaStream_t s);
+                          cudaStream_t s, float* copy = nullptr);
 cudaError_t launch_sample(dflare_ctx* c, int rows, float inv_t, uint64_t seed, const uint64_t* step,
-                          int32_t* tokens, cudaStream_t s);
+                          int32_t* tokens, cudaStream_t s, float* copy = nullptr);
 cudaError_t launch_spec_stats(dflare_ctx* c, const float* target_logits, float inv_t, cudaStream_t s);
 cudaError_t launch_spec_accept(dflare_ctx* c, const int32_t* draft, const float* target_logits,
                                float inv_t, uint64_t seed, const uint64_t* step, cudaStream_t s);

@@ -131,14 +131,25 @@ __device__ __forceinline__ void load4(const float* p, int i, int c1, bool vec, f
     }
 }
 
+__device__ __forceinline__ void store4(float* p, int i, int c1, bool vec, const float* x) {
+    if (vec && i + 4 <= c1) {
+        *reinterpret_cast<float4*>(p + i) = make_float4(x[0], x[1], x[2], x[3]);
+    } else {
+#pragma unroll
+        for (int e = 0; e < 4; ++e)
+            if (i + e < c1) p[i + e] = x[e];
+    }
+}
+
 // ---------------------------------------------------------------------------------- drafting
 // Grid (chunks, rows), chunk a multiple of 8: every thread takes groups of eight logits and the
-// one Philox block that covers them.
+// one Philox block that covers them. copy (when given) receives the logits as they are read.
 __global__ void __launch_bounds__(256) sample_kernel(const float* __restrict__ logits, int V, int rows,
                                                      int chunk, float inv_t, uint64_t seed,
                                                      const uint64_t* __restrict__ step_dev,
                                                      unsigned long long* slot, uint32_t* cnt,
-                                                     int32_t* __restrict__ tokens) {
+                                                     int32_t* __restrict__ tokens,
+                                                     float* __restrict__ copy) {
     pdl_trigger();
     pdl_wait();
     const uint64_t step = *step_dev;
@@ -146,6 +157,7 @@ __global__ void __launch_bounds__(256) sample_kernel(const float* __restrict__ l
     const int c0 = blockIdx.x * chunk, c1 = min(V, c0 + chunk);
     const float* p = logits + (size_t)row * V;
     const bool vec = (V & 3) == 0;
+    float* const cp = copy ? copy + (size_t)row * V : nullptr;
     float bv = -INFINITY;
     int bi = kNone;
     // kDrawU groups of eight logits (one Philox block each) per thread and iteration, all loads
@@ -163,6 +175,10 @@ __global__ void __launch_bounds__(256) sample_kernel(const float* __restrict__ l
         for (int g = 0; g < kDrawU; ++g) {
             const int i = base + g * stride;
             if (i >= c1) break;
+            if (cp) {
+                store4(cp, i, c1, vec, x[g]);
+                store4(cp, i + 4, c1, vec, x[g] + 4);
+            }
             float u[8];
             philox_uniforms(1 + (uint64_t)(i >> 3), (uint64_t)row, step, kRngDraft, seed, u);
 #pragma unroll
@@ -414,13 +430,13 @@ void chunking(int V, int rows, int sms, int max_chunks, int per_sm, int* chunk, 
 }  // namespace
 
 cudaError_t launch_sample(dflare_ctx* c, int rows, float inv_t, uint64_t seed, const uint64_t* step,
-                          int32_t* tokens, cudaStream_t s) {
+                          int32_t* tokens, cudaStream_t s, float* copy) {
     if (rows <= 0) return cudaSuccess;
     int chunk, chunks;
     chunking(c->cfg.vocab, rows, c->num_sms, 1 << 20, 4, &chunk, &chunks);
     return launch_kernel(c->pdl, sample_kernel, dim3(chunks, rows), dim3(256), 0, s, c->logits,
                          c->cfg.vocab, rows, chunk, inv_t, seed, step, c->amax_slot, c->amax_cnt,
-                         tokens);
+                         tokens, copy);
 }
 
 cudaError_t launch_spec_stats(dflare_ctx* c, const float* target_logits, float inv_t, cudaStream_t s) {

@@ -15,11 +15,13 @@ namespace {
 // first layer's normalised input RMSNorm(X^0) in the storage type.
 // qkv32 (when given, n32 floats per block row) is cleared here, at the start of every drafted
 // block, so that the first layer's Q/K^d/V^d reductions start from zero even after an aborted call.
+// copy (when given): a second copy of X^0, the caller's hidden states before the first layer.
 template <class T>
 __global__ void embed_kernel(const T* __restrict__ E, const int32_t* __restrict__ last_token,
                              int mask_id, int V, int B, int d, float* __restrict__ X,
                              T* __restrict__ Xn, const T* __restrict__ gain, float eps,
-                             uint32_t* err, float* __restrict__ qkv32, int n32) {
+                             uint32_t* err, float* __restrict__ qkv32, int n32,
+                             float* __restrict__ copy) {
     pdl_trigger();
     pdl_wait();
     __shared__ float red[32];
@@ -41,6 +43,7 @@ __global__ void embed_kernel(const T* __restrict__ E, const int32_t* __restrict_
     if (act) {
         load8(E + (size_t)tok * d + e0, v);
         store8(X + row * d + e0, v);
+        if (copy) store8(copy + row * d + e0, v);
 #pragma unroll
         for (int e = 0; e < 8; ++e) ss = fmaf(v[e], v[e], ss);
     }
@@ -58,11 +61,13 @@ __global__ void embed_kernel(const T* __restrict__ E, const int32_t* __restrict_
 // out[r] = gain * X[row(r)] / sqrt(mean(X^2) + eps). With `gather`, output row r reads the mask
 // row k = r % (B-1) + 1 of sequence r / (B-1) (the LM head only needs the mask positions). With
 // zero32, row r of it (n32 floats) is cleared: the fp32 sums the next Q/K^d/V^d projection adds
-// into (the previous layer's attention, which read them, is complete by now).
+// into (the previous layer's attention, which read them, is complete by now). With copy, the rows of
+// X go there as well (the caller's hidden states after the previous layer); a gather then runs over
+// all block rows, of which the first of each sequence is only copied.
 template <class T>
 __global__ void rmsnorm_kernel(const float* __restrict__ X, const T* __restrict__ gain,
                                T* __restrict__ out, int d, int B, int gather, float eps,
-                               float* __restrict__ zero32, int n32) {
+                               float* __restrict__ zero32, int n32, float* __restrict__ copy) {
     pdl_trigger();
     const int e0 = threadIdx.x * 8;
     const bool act = e0 < d;
@@ -75,11 +80,19 @@ __global__ void rmsnorm_kernel(const float* __restrict__ X, const T* __restrict_
         float4* z = reinterpret_cast<float4*>(zero32 + (size_t)r * n32);
         for (int i = threadIdx.x; i < n32 / 4; i += blockDim.x) z[i] = make_float4(0.f, 0.f, 0.f, 0.f);
     }
-    const size_t in_row = gather ? (size_t)(r / (B - 1)) * B + (r % (B - 1)) + 1 : (size_t)r;
+    size_t in_row = r, out_row = r;
+    if (gather && copy)
+        out_row = (size_t)(r / B) * (B - 1) + r % B - 1;   // (not used for the first row of a block)
+    else if (gather)
+        in_row = (size_t)(r / (B - 1)) * B + (r % (B - 1)) + 1;
     float v[8];
     float ss = 0.f;
     if (act) {
         load8(X + in_row * d + e0, v);
+        if (copy) store8(copy + in_row * d + e0, v);
+    }
+    if (gather && copy && r % B == 0) return;
+    if (act) {
 #pragma unroll
         for (int e = 0; e < 8; ++e) ss = fmaf(v[e], v[e], ss);
     }
@@ -89,7 +102,7 @@ __global__ void rmsnorm_kernel(const float* __restrict__ X, const T* __restrict_
         float o[8];
 #pragma unroll
         for (int e = 0; e < 8; ++e) o[e] = g[e] * (v[e] * inv);
-        store8(out + (size_t)r * d + e0, o);
+        store8(out + out_row * d + e0, o);
     }
 }
 
@@ -105,11 +118,13 @@ __device__ __forceinline__ uint32_t ordered_key(float v) {
 // 64-bit atomicMax; the last CTA to finish turns the packed maxima into token ids and re-arms
 // the slots and the counter for the next launch. NaN entries are never chosen. A row without a
 // value above -inf publishes nothing; the last CTA then takes its first -inf entry (the lowest
-// id among equal maxima), or id 0 when every entry is NaN.
+// id among equal maxima), or id 0 when every entry is NaN. copy (when given) receives the logits as
+// they are read (16-byte aligned when V is a multiple of 4): the caller's copy costs no second pass.
 __global__ void __launch_bounds__(256) argmax_kernel(const float* __restrict__ logits, int V,
                                                      int rows, int chunk,
                                                      unsigned long long* slot, uint32_t* cnt,
-                                                     int32_t* __restrict__ tokens) {
+                                                     int32_t* __restrict__ tokens,
+                                                     float* __restrict__ copy) {
     pdl_trigger();
     pdl_wait();
     __shared__ float sv[8];
@@ -118,6 +133,7 @@ __global__ void __launch_bounds__(256) argmax_kernel(const float* __restrict__ l
     const int row = blockIdx.y;
     const int c0 = blockIdx.x * chunk, c1 = min(V, c0 + chunk);
     const float* p = logits + (size_t)row * V;
+    float* const cp = copy ? copy + (size_t)row * V : nullptr;
     float bv = -INFINITY;
     int bi = 0x7fffffff;
     if ((V & 3) == 0) {
@@ -137,6 +153,7 @@ __global__ void __launch_bounds__(256) argmax_kernel(const float* __restrict__ l
 #pragma unroll
             for (int u = 0; u < U; ++u) {
                 const int i = base + u * stride;
+                if (cp && i < c1) *reinterpret_cast<float4*>(cp + i) = q[u];
                 if (q[u].x > bv) { bv = q[u].x; bi = i; }
                 if (q[u].y > bv) { bv = q[u].y; bi = i + 1; }
                 if (q[u].z > bv) { bv = q[u].z; bi = i + 2; }
@@ -146,6 +163,7 @@ __global__ void __launch_bounds__(256) argmax_kernel(const float* __restrict__ l
     } else {
         for (int i = c0 + threadIdx.x; i < c1; i += blockDim.x) {
             const float q = p[i];
+            if (cp) cp[i] = q;
             if (q > bv) { bv = q; bi = i; }
         }
     }
@@ -231,37 +249,38 @@ __global__ void synth_target_kernel(const int32_t* __restrict__ draft, const uin
 
 }  // namespace
 
-cudaError_t launch_embed(dflare_ctx* c, const int32_t* last_token, cudaStream_t s) {
+cudaError_t launch_embed(dflare_ctx* c, const int32_t* last_token, cudaStream_t s, float* copy) {
     const dflare_config& g = c->cfg;
     const dim3 grid(g.block, c->batch), block(((g.d / 8 + 31) / 32) * 32);
     if (g.dtype == DFLARE_F32)
         return launch_kernel(c->pdl, embed_kernel<float>, grid, block, 0, s,
                              (const float*)c->w.embed, last_token, g.mask_token_id, g.vocab, g.block,
                              g.d, c->x, (float*)c->xn, (const float*)c->w.attn_norm, g.rms_eps,
-                             c->err, (float*)nullptr, 0);
+                             c->err, (float*)nullptr, 0, copy);
     return launch_kernel(c->pdl, embed_kernel<bf16>, grid, block, 0, s, (const bf16*)c->w.embed,
                          last_token, g.mask_token_id, g.vocab, g.block, g.d, c->x, (bf16*)c->xn,
                          (const bf16*)c->w.attn_norm, g.rms_eps, c->err, c->qkv32,
-                         (g.n_q_heads + 2 * g.n_kv_heads) * g.head_dim);
+                         (g.n_q_heads + 2 * g.n_kv_heads) * g.head_dim, copy);
 }
 
 cudaError_t launch_rmsnorm(dflare_ctx* c, const void* gain, int rows, bool gather, void* out,
-                           cudaStream_t s, float* zero32) {
+                           cudaStream_t s, float* zero32, float* copy) {
     const dflare_config& g = c->cfg;
     if (rows <= 0) return cudaSuccess;
+    if (gather && copy) rows = c->batch * g.block;
     const dim3 block(((g.d / 8 + 31) / 32) * 32);
     const int n32 = (g.n_q_heads + 2 * g.n_kv_heads) * g.head_dim;
     if (g.dtype == DFLARE_F32)
         return launch_kernel(c->pdl, rmsnorm_kernel<float>, dim3(rows), block, 0, s, c->x,
                              (const float*)gain, (float*)out, g.d, g.block, gather ? 1 : 0,
-                             g.rms_eps, zero32, n32);
+                             g.rms_eps, zero32, n32, copy);
     return launch_kernel(c->pdl, rmsnorm_kernel<bf16>, dim3(rows), block, 0, s, c->x,
                          (const bf16*)gain, (bf16*)out, g.d, g.block, gather ? 1 : 0, g.rms_eps,
-                         zero32, n32);
+                         zero32, n32, copy);
 }
 
 cudaError_t launch_argmax(dflare_ctx* c, const float* logits, int rows, int32_t* tokens,
-                          cudaStream_t s) {
+                          cudaStream_t s, float* copy) {
     if (rows <= 0) return cudaSuccess;
     const int V = c->cfg.vocab;
     // about four CTAs per SM (measured against two: 0.5207 -> 0.5195 ms per Qwen3-4B-shaped step;
@@ -271,7 +290,7 @@ cudaError_t launch_argmax(dflare_ctx* c, const float* logits, int rows, int32_t*
     chunk = std::max(4096, ((chunk + 1023) / 1024) * 1024);
     chunks = (V + chunk - 1) / chunk;
     return launch_kernel(c->pdl, argmax_kernel, dim3(chunks, rows), dim3(256), 0, s, logits, V,
-                         rows, chunk, c->amax_slot, c->amax_cnt, tokens);
+                         rows, chunk, c->amax_slot, c->amax_cnt, tokens, copy);
 }
 
 cudaError_t launch_verify(dflare_ctx* c, const int32_t* draft, const int32_t* target,

@@ -60,3 +60,31 @@ def test_simt_gemm_on_bf16_matches_oracle():
     """The CUDA-core GEMM on bf16 weights (a cross-check of the tensor-core GEMM)."""
     from paper_2606_02091_gb300 import FLAG_SIMT_GEMM
     _step_matches_oracle(synth.Workload("simt_bf16", _shape(d=320, ffn=192, vocab=333, block=9), (40, 3), 0.8, 35), FLAG_SIMT_GEMM)
+
+
+@pytest.mark.parametrize("vocab,block,sampled", [(1000, 8, False), (1003, 8, False), (1000, 8, True), (1003, 5, True), (300, 1, False)])
+def test_copies_to_aligned_and_unaligned_buffers_agree(vocab, block, sampled):
+    """logits_out and hidden_out as written by the kernels (16-byte aligned buffers) and as copied
+    afterwards (buffers 4 bytes further) hold the same bits; the deterministic mode repeats exactly."""
+    import torch
+    from paper_2606_02091_gb300 import FLAG_DETERMINISTIC
+    w = synth.Workload("copies", _shape(vocab=vocab, block=block), (33, 70), 0.8, 36)
+    g = GpuSide(w, flags=FLAG_DETERMINISTIC)
+    g.fuse(w.ctx_lens, want_fused=False)
+    s = w.shape
+    last = torch.tensor(synth.initial_tokens(w), device="cuda")
+    step = torch.zeros(1, dtype=torch.int64, device="cuda")
+    got = []
+    for off in (0, 1):
+        toks = torch.zeros((w.batch, block - 1), dtype=torch.int32, device="cuda")
+        logits = torch.zeros(w.batch * (block - 1) * vocab + 4, dtype=torch.float32, device="cuda")[off:]
+        hidden = torch.zeros((s.n_draft_layers + 1) * w.batch * block * s.d + 4, dtype=torch.float32, device="cuda")[off:]
+        if sampled:
+            g.lib.draft_block_sampled(last, 1.0, 7, step, toks, logits, hidden)
+        else:
+            g.lib.draft_block(last, toks, logits, hidden)
+        torch.cuda.synchronize()
+        got.append([t.cpu().numpy() for t in (toks, logits[:w.batch * (block - 1) * vocab], hidden[:(s.n_draft_layers + 1) * w.batch * block * s.d])])
+        assert got[-1][2].any() and (block == 1 or got[-1][1].all())
+    for a, b in zip(*got):
+        np.testing.assert_array_equal(a, b)
