@@ -298,7 +298,7 @@ dflare_status dflare_device_error(dflare_ctx* ctx, uint32_t* bits_host, void* st
  * `stream` (name: "fuse_begin", "fuse_layers", "gemm_fusion_fc", "gemm_dflash_fc",
  * "gemm_kv_ctx", "embed", "rmsnorm", "gemm_qkv",
  * "attention", "gemm_o", "gemm_gate_up", "gemm_down", "gemm_lm_head", "argmax", "sample",
- * "argmax_target", "verify", "spec_stats", "spec_accept", "spec_resample").
+ * "argmax_target" (with the acceptance), "verify", "spec_stats", "spec_resample").
  * A caller can record CUDA events there, also while the stream is being captured into a graph.
  * fn = NULL turns tracing off. */
 typedef void (*dflare_trace_fn)(void* user, const char* name, int phase, void* stream);

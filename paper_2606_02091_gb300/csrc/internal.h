@@ -251,13 +251,14 @@ cudaError_t launch_attention(dflare_ctx* c, int layer, cudaStream_t s);
 // copy (optional, 16-byte aligned): receives the logits, [rows][V]
 cudaError_t launch_argmax(dflare_ctx* c, const float* logits, int rows, int32_t* tokens,
                           cudaStream_t s, float* copy = nullptr);
+// launch_argmax over the target's logits [batch*B][V], then launch_verify's decisions in its last CTA
+cudaError_t launch_argmax_verify(dflare_ctx* c, const float* target_logits, const int32_t* draft,
+                                 int32_t* accept_len, int32_t* next_token, cudaStream_t s);
 cudaError_t launch_sample(dflare_ctx* c, int rows, float inv_t, uint64_t seed, const uint64_t* step,
                           int32_t* tokens, cudaStream_t s, float* copy = nullptr);
 cudaError_t launch_spec_stats(dflare_ctx* c, const float* target_logits, float inv_t, cudaStream_t s);
-cudaError_t launch_spec_accept(dflare_ctx* c, const int32_t* draft, const float* target_logits,
-                               float inv_t, uint64_t seed, const uint64_t* step, cudaStream_t s);
-cudaError_t launch_spec_resample(dflare_ctx* c, const float* target_logits, float inv_t,
-                                 uint64_t seed, uint64_t* step, int32_t* accept_len,
+cudaError_t launch_spec_resample(dflare_ctx* c, const int32_t* draft, const float* target_logits,
+                                 float inv_t, uint64_t seed, uint64_t* step, int32_t* accept_len,
                                  int32_t* next_token, cudaStream_t s);
 cudaError_t launch_verify(dflare_ctx* c, const int32_t* draft, const int32_t* target,
                           int32_t* accept_len, int32_t* next_token, cudaStream_t s);

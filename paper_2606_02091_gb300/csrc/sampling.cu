@@ -275,72 +275,94 @@ __global__ void __launch_bounds__(256) spec_stats_kernel(const float* __restrict
     }
 }
 
-// (max, normaliser) of one row from its chunk partials
-__device__ __forceinline__ float2 row_stats(const float2* part, int row, int chunks) {
-    float m = -INFINITY, s = 0.f;
-#pragma unroll 8
-    for (int c = 0; c < chunks; ++c) {
-        const float2 q = part[(size_t)row * chunks + c];
-        const float M = fmaxf(m, q.x);
-        if (M > -INFINITY)
-            s = (m > -INFINITY ? s * expf(m - M) : 0.f) + (q.x > -INFINITY ? q.y * expf(q.x - M) : 0.f);
-        m = M;
-    }
-    return make_float2(m, s);
+// (m, s) merged with another chunk's partial (m = -inf: nothing above -inf in it)
+__device__ __forceinline__ void merge_stats(float& m, float& s, float2 q) {
+    const float M = fmaxf(m, q.x);
+    if (M > -INFINITY)
+        s = (m > -INFINITY ? s * expf(m - M) : 0.f) + (q.x > -INFINITY ? q.y * expf(q.x - M) : 0.f);
+    m = M;
 }
 
-// One warp per sequence: lane j decides draft token d_{j+1} (target row j, draft row j, uniform
-// j of the acceptance stream); a = the first rejected position (B-1 when none) goes to spec_a.
-__global__ void __launch_bounds__(32) spec_accept_kernel(const float* __restrict__ target,
-                                                         const float* __restrict__ draft_logits,
-                                                         const int32_t* __restrict__ draft, int V,
-                                                         int B, int batch, int chunks, float inv_t,
-                                                         uint64_t seed, const uint64_t* __restrict__ step_dev,
-                                                         const float2* __restrict__ part,
-                                                         int32_t* __restrict__ spec_a, uint32_t* err) {
-    pdl_trigger();
-    pdl_wait();
-    const int b = blockIdx.x, j = threadIdx.x;
-    const uint64_t step = *step_dev;
-    bool rej = false;
-    if (j < B - 1) {
-        const int d = draft[(size_t)b * (B - 1) + j];
-        if (d < 0 || d >= V) {
-            rej = true;
-            atomicOr(err, DFLARE_DEVERR_TOKEN);
+// Softmax statistics of sequence b's rows and its first rejected draft position, computed by every
+// CTA of the sequence (256 threads) for itself: the partials and B - 1 gathered logits are a few
+// KB from L2, less than the launch of a kernel that would leave them ready. Warps 0, 2, 4, 6 merge
+// the chunk partials of target row `lane` (a quarter of the chunks each), warps 1, 3, 5, 7 those of
+// draft row `lane`; lane j of warp 0 then decides draft token d_{j+1} (target row j, draft row j,
+// uniform j of the acceptance stream).
+struct Accept {
+    float2 part[2][4][32];
+    float2 stat[2][32];   // target rows 0 .. B-1, draft rows 0 .. B-2
+    int a;                // the first rejected position, B - 1 when none
+};
+__device__ __forceinline__ void accept_block(Accept& sh, const float* target, const float* draft_logits,
+                                             const int32_t* draft, int V, int B, int batch, int chunks,
+                                             float inv_t, uint64_t seed, uint64_t step, const float2* part,
+                                             int b, uint32_t* err) {
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    const int kind = warp & 1, quarter = warp >> 1;
+    float lt = 0.f, lq = 0.f, u = 0.f;
+    bool valid = false;
+    if (warp == 0 && lane < B - 1) {
+        const int d = draft[(size_t)b * (B - 1) + lane];
+        valid = d >= 0 && d < V;
+        if (valid) {
+            lt = target[(size_t)(b * B + lane) * V + d] * inv_t;
+            lq = draft_logits[(size_t)(b * (B - 1) + lane) * V + d] * inv_t;
         } else {
-            const int tr = b * B + j, dr = b * (B - 1) + j;
-            const float2 st = row_stats(part, tr, chunks);
-            const float2 sq = row_stats(part, batch * B + dr, chunks);
-            const float p = expf(target[(size_t)tr * V + d] * inv_t - st.x) / st.y;
-            const float q = expf(draft_logits[(size_t)dr * V + d] * inv_t - sq.x) / sq.y;
-            float u[8];
-            philox_uniforms(1 + (uint64_t)(j >> 3), (uint64_t)b, step, kRngAccept, seed, u);
-            rej = !(u[j & 7] * q < p);
+            atomicOr(err, DFLARE_DEVERR_TOKEN);
         }
     }
-    const unsigned mask = __ballot_sync(0xffffffffu, rej);
-    if (j == 0) spec_a[b] = mask ? __ffs(mask) - 1 : B - 1;
+    float m = -INFINITY, s = 0.f;
+    if (lane < B - kind) {
+        const float2* p = part + (size_t)(kind ? batch * B + b * (B - 1) + lane : b * B + lane) * chunks;
+#pragma unroll 4
+        for (int c = quarter; c < chunks; c += 4) merge_stats(m, s, p[c]);
+    }
+    sh.part[kind][quarter][lane] = make_float2(m, s);
+    if (warp == 0 && valid) {
+        float v[8];
+        philox_uniforms(1 + (uint64_t)(lane >> 3), (uint64_t)b, step, kRngAccept, seed, v);
+#pragma unroll
+        for (int e = 0; e < 8; ++e)
+            if (e == (lane & 7)) u = v[e];
+    }
+    __syncthreads();
+    if (warp < 2) {
+        for (int q = 1; q < 4; ++q) merge_stats(m, s, sh.part[warp][q][lane]);
+        sh.stat[warp][lane] = make_float2(m, s);
+    }
+    __syncthreads();
+    if (warp == 0) {
+        const float2 sq = sh.stat[1][lane];
+        const float p = expf(lt - m) / s, q = expf(lq - sq.x) / sq.y;
+        const unsigned rej = __ballot_sync(0xffffffffu, lane < B - 1 && !(valid && u * q < p));
+        if (lane == 0) sh.a = rej ? __ffs(rej) - 1 : B - 1;
+    }
+    __syncthreads();
 }
 
-// Grid (chunks, batch): the replacement draw of every sequence, from max(0, p - q) at its first
-// rejected position a, or from p at the last target row when every draft was kept. The last CTA
-// writes accept_len = a + 1 and the token, re-arms the slots, and advances the step counter.
+// Grid (chunks, batch): the acceptance decisions and the replacement draw of every sequence, from
+// max(0, p - q) at its first rejected position a, or from p at the last target row when every draft
+// was kept. The last CTA writes accept_len = a + 1 and the token, re-arms the slots, and advances the
+// step counter.
 __global__ void __launch_bounds__(256) spec_resample_kernel(
-    const float* __restrict__ target, const float* __restrict__ draft_logits, int V, int B,
-    int batch, int chunk, int stat_chunks, float inv_t, uint64_t seed, uint64_t* step_dev,
-    const float2* __restrict__ part, const int32_t* __restrict__ spec_a,
+    const float* __restrict__ target, const float* __restrict__ draft_logits,
+    const int32_t* __restrict__ draft, int V, int B, int batch, int chunk, int stat_chunks, float inv_t,
+    uint64_t seed, uint64_t* step_dev, const float2* __restrict__ part, int32_t* spec_a,
     unsigned long long* slot, uint32_t* cnt, int32_t* __restrict__ accept_len,
-    int32_t* __restrict__ next_token) {
+    int32_t* __restrict__ next_token, uint32_t* err) {
     pdl_trigger();
+    __shared__ Accept sh;
     pdl_wait();
     const uint64_t step = *step_dev;
     const int b = blockIdx.y;
-    const int a = spec_a[b];
+    accept_block(sh, target, draft_logits, draft, V, B, batch, stat_chunks, inv_t, seed, step, part, b, err);
+    const int a = sh.a;
     const bool resid = a < B - 1;
     const int tr = b * B + a, dr = b * (B - 1) + a;
-    const float2 st = row_stats(part, tr, stat_chunks);
-    const float2 sq = resid ? row_stats(part, batch * B + dr, stat_chunks) : make_float2(0.f, 1.f);
+    const float2 st = sh.stat[0][a];
+    const float2 sq = resid ? sh.stat[1][a] : make_float2(0.f, 1.f);
+    if (blockIdx.x == 0 && threadIdx.x == 0) spec_a[b] = a;   // for the last CTA (fenced in publish_max)
     const float* lt = target + (size_t)tr * V;
     const float* lq = resid ? draft_logits + (size_t)dr * V : nullptr;
     const int c0 = blockIdx.x * chunk, c1 = min(V, c0 + chunk);
@@ -382,13 +404,14 @@ __global__ void __launch_bounds__(256) spec_resample_kernel(
     if (publish_max(bv, bi, &slot[b], cnt, gridDim.x * gridDim.y)) {
         for (int s = threadIdx.x; s < batch; s += blockDim.x) {
             const unsigned long long key = atomicExch(&slot[s], 0ull);
-            const int as = spec_a[s];
+            const int as = __ldcg(spec_a + s);
             int32_t tok = slot_token(key);
             if (key == 0ull) {
                 // max(0, p - q) vanished everywhere (or every entry was -inf): draw from p at
                 // that target row instead, serially (only for such rows)
                 const int r = s * B + as;
-                const float2 t2 = row_stats(part, r, stat_chunks);
+                float2 t2 = make_float2(-INFINITY, 0.f);
+                for (int c = 0; c < stat_chunks; ++c) merge_stats(t2.x, t2.y, part[(size_t)r * stat_chunks + c]);
                 const float* l = target + (size_t)r * V;
                 float best = -INFINITY;
                 tok = 0;
@@ -450,24 +473,16 @@ cudaError_t launch_spec_stats(dflare_ctx* c, const float* target_logits, float i
                          c->spec_part);
 }
 
-cudaError_t launch_spec_accept(dflare_ctx* c, const int32_t* draft, const float* target_logits,
-                               float inv_t, uint64_t seed, const uint64_t* step, cudaStream_t s) {
-    return launch_kernel(c->pdl, spec_accept_kernel, dim3(c->batch), dim3(32), 0, s, target_logits,
-                         (const float*)c->logits, draft, c->cfg.vocab, c->cfg.block, c->batch,
-                         c->spec_chunks, inv_t, seed, step, (const float2*)c->spec_part, c->spec_a,
-                         c->err);
-}
-
-cudaError_t launch_spec_resample(dflare_ctx* c, const float* target_logits, float inv_t,
-                                 uint64_t seed, uint64_t* step, int32_t* accept_len,
+cudaError_t launch_spec_resample(dflare_ctx* c, const int32_t* draft, const float* target_logits,
+                                 float inv_t, uint64_t seed, uint64_t* step, int32_t* accept_len,
                                  int32_t* next_token, cudaStream_t s) {
     int chunk, chunks;
     chunking(c->cfg.vocab, c->batch, c->num_sms, 1 << 20, 2, &chunk, &chunks);
     return launch_kernel(c->pdl, spec_resample_kernel, dim3(chunks, c->batch), dim3(256), 0, s,
-                         target_logits, (const float*)c->logits, c->cfg.vocab, c->cfg.block,
+                         target_logits, (const float*)c->logits, draft, c->cfg.vocab, c->cfg.block,
                          c->batch, chunk, c->spec_chunks, inv_t, seed, step,
-                         (const float2*)c->spec_part, (const int32_t*)c->spec_a, c->amax_slot,
-                         c->amax_cnt, accept_len, next_token);
+                         (const float2*)c->spec_part, c->spec_a, c->amax_slot, c->amax_cnt, accept_len,
+                         next_token, c->err);
 }
 
 }  // namespace dfl

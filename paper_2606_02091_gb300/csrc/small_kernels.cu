@@ -113,6 +113,30 @@ __device__ __forceinline__ uint32_t ordered_key(float v) {
     return (u & 0x80000000u) ? ~u : (u | 0x80000000u);
 }
 
+// Prefix acceptance (Sec. 3.2, verification) of sequence b by one warp: lane l compares d_{l+1}
+// with g_l, the first mismatch ends the accepted prefix.
+__device__ __forceinline__ void accept_prefix(const int32_t* draft, const int32_t* target, int32_t* accept_len,
+                                              int32_t* next_token, int b, int B) {
+    const int lane = threadIdx.x & 31;
+    bool mism = false;
+    if (lane < B - 1) mism = draft[(size_t)b * (B - 1) + lane] != target[(size_t)b * B + lane];
+    const unsigned m = __ballot_sync(0xffffffffu, mism);
+    const int a = m ? __ffs(m) - 1 : B - 1;
+    if (lane == 0) {
+        accept_len[b] = a + 1;
+        next_token[b] = target[(size_t)b * B + a];
+    }
+}
+
+__global__ void verify_kernel(const int32_t* __restrict__ draft, const int32_t* __restrict__ target,
+                              int32_t* __restrict__ accept_len, int32_t* __restrict__ next_token,
+                              int batch, int B) {
+    pdl_trigger();
+    pdl_wait();
+    const int b = blockIdx.x * (blockDim.x >> 5) + (threadIdx.x >> 5);
+    if (b < batch) accept_prefix(draft, target, accept_len, next_token, b, B);
+}
+
 // Greedy argmax over the vocabulary (lowest id among equal maxima). Grid (chunks, rows): each
 // CTA reduces a chunk of one row with warp shuffles and publishes (key(value), ~index) through a
 // 64-bit atomicMax; the last CTA to finish turns the packed maxima into token ids and re-arms
@@ -120,11 +144,15 @@ __device__ __forceinline__ uint32_t ordered_key(float v) {
 // value above -inf publishes nothing; the last CTA then takes its first -inf entry (the lowest
 // id among equal maxima), or id 0 when every entry is NaN. copy (when given) receives the logits as
 // they are read (16-byte aligned when V is a multiple of 4): the caller's copy costs no second pass.
+// With accept_len, the rows are a target's [batch][B] and the last CTA goes on to the acceptance of
+// the drafts.
 __global__ void __launch_bounds__(256) argmax_kernel(const float* __restrict__ logits, int V,
                                                      int rows, int chunk,
                                                      unsigned long long* slot, uint32_t* cnt,
-                                                     int32_t* __restrict__ tokens,
-                                                     float* __restrict__ copy) {
+                                                     int32_t* tokens, float* __restrict__ copy,
+                                                     const int32_t* __restrict__ draft, int B,
+                                                     int32_t* __restrict__ accept_len,
+                                                     int32_t* __restrict__ next_token) {
     pdl_trigger();
     pdl_wait();
     __shared__ float sv[8];
@@ -203,26 +231,11 @@ __global__ void __launch_bounds__(256) argmax_kernel(const float* __restrict__ l
             tokens[r] = tok;
         }
         if (threadIdx.x == 0) *cnt = 0;
-    }
-}
-
-// Prefix acceptance (Sec. 3.2, verification): one warp per sequence; lane l compares d_{l+1}
-// with g_l, the first mismatch ends the accepted prefix.
-__global__ void verify_kernel(const int32_t* __restrict__ draft, const int32_t* __restrict__ target,
-                              int32_t* __restrict__ accept_len, int32_t* __restrict__ next_token,
-                              int batch, int B) {
-    pdl_trigger();
-    pdl_wait();
-    const int lane = threadIdx.x & 31;
-    const int b = blockIdx.x * (blockDim.x >> 5) + (threadIdx.x >> 5);
-    if (b >= batch) return;
-    bool mism = false;
-    if (lane < B - 1) mism = draft[(size_t)b * (B - 1) + lane] != target[(size_t)b * B + lane];
-    const unsigned m = __ballot_sync(0xffffffffu, mism);
-    const int a = m ? __ffs(m) - 1 : B - 1;
-    if (lane == 0) {
-        accept_len[b] = a + 1;
-        next_token[b] = target[(size_t)b * B + a];
+        if (accept_len) {
+            __syncthreads();   // every row's token is written
+            for (int b = threadIdx.x >> 5; b < rows / B; b += blockDim.x >> 5)
+                accept_prefix(draft, tokens, accept_len, next_token, b, B);
+        }
     }
 }
 
@@ -279,8 +292,8 @@ cudaError_t launch_rmsnorm(dflare_ctx* c, const void* gain, int rows, bool gathe
                          zero32, n32, copy);
 }
 
-cudaError_t launch_argmax(dflare_ctx* c, const float* logits, int rows, int32_t* tokens,
-                          cudaStream_t s, float* copy) {
+static cudaError_t run_argmax(dflare_ctx* c, const float* logits, int rows, int32_t* tokens, cudaStream_t s,
+                              float* copy, const int32_t* draft, int32_t* accept_len, int32_t* next_token) {
     if (rows <= 0) return cudaSuccess;
     const int V = c->cfg.vocab;
     // about four CTAs per SM (measured against two: 0.5207 -> 0.5195 ms per Qwen3-4B-shaped step;
@@ -290,7 +303,18 @@ cudaError_t launch_argmax(dflare_ctx* c, const float* logits, int rows, int32_t*
     chunk = std::max(4096, ((chunk + 1023) / 1024) * 1024);
     chunks = (V + chunk - 1) / chunk;
     return launch_kernel(c->pdl, argmax_kernel, dim3(chunks, rows), dim3(256), 0, s, logits, V,
-                         rows, chunk, c->amax_slot, c->amax_cnt, tokens, copy);
+                         rows, chunk, c->amax_slot, c->amax_cnt, tokens, copy, draft, c->cfg.block, accept_len,
+                         next_token);
+}
+
+cudaError_t launch_argmax(dflare_ctx* c, const float* logits, int rows, int32_t* tokens,
+                          cudaStream_t s, float* copy) {
+    return run_argmax(c, logits, rows, tokens, s, copy, nullptr, nullptr, nullptr);
+}
+
+cudaError_t launch_argmax_verify(dflare_ctx* c, const float* target_logits, const int32_t* draft,
+                                 int32_t* accept_len, int32_t* next_token, cudaStream_t s) {
+    return run_argmax(c, target_logits, c->batch * c->cfg.block, c->tgt_tok, s, nullptr, draft, accept_len, next_token);
 }
 
 cudaError_t launch_verify(dflare_ctx* c, const int32_t* draft, const int32_t* target,
