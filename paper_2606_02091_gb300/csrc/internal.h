@@ -74,6 +74,7 @@ struct GemmDesc {
     int max_smem = 0;      // tcgen05 GEMM: shared-memory budget per CTA in bytes (0 = default)
     int evict_first = 0;   // tcgen05 GEMM: weights with an L2 evict-first policy (0 = yes, -1 = no)
     int force_splits = 0;  // tcgen05 GEMM: K splits (0 = chosen from the wave count)
+    int force_bn = 0;      // two-SM GEMM: features per tile (0 = chosen from the cost model)
 };
 
 }  // namespace dfl
@@ -236,6 +237,9 @@ int attention_launch_splits(const dflare_ctx* c);
 // strides_bytes for dims 1..rank-1); false when the driver rejects it.
 bool encode_tma_bf16(CUtensorMap* m, const void* base, int rank, const uint64_t* dims,
                      const uint64_t* strides_bytes, const uint32_t* box);
+// the same over fp32 elements
+bool encode_tma_f32(CUtensorMap* m, const void* base, int rank, const uint64_t* dims,
+                    const uint64_t* strides_bytes, const uint32_t* box);
 cudaError_t launch_gemm_simt(dflare_ctx* c, const GemmDesc& g, cudaStream_t s);
 cudaError_t launch_fusion_alpha(dflare_ctx* c, cudaStream_t s);
 cudaError_t launch_fuse_begin(dflare_ctx* c, const int32_t* n_new, int n_max, cudaStream_t s);
