@@ -107,7 +107,7 @@ dflare_status gemm(dflare_ctx* c, const GemmDesc& g, cudaStream_t s) {
     cudaError_t e;
     std::string why;
     if (use_tc(c))
-        e = launch_gemm_tc(c, g, s, &why);
+        e = gemm_pair_fits(c, g) ? launch_gemm_pair(c, g, s, &why) : launch_gemm_tc(c, g, s, &why);
     else
         e = launch_gemm_simt(c, g, s);
     if (e != cudaSuccess)

@@ -8,8 +8,7 @@
 // the UMMA N dimension (16..256), so one instruction covers a 128 x bn x 16 piece.
 //
 // Work unit = (group, 128-feature tile, token tile, K split); for an LM head over 128+ token rows,
-// a pair of adjacent 128-feature tiles (two accumulators over one activation tile); a context
-// fill's units run only over the token tiles that hold appended rows. A
+// a pair of adjacent 128-feature tiles (two accumulators over one activation tile). A
 // persistent grid of one CTA per SM walks the units. Per CTA (192 threads):
 //   warp 4    TMA producer: per stage, kbs consecutive 128x64 bf16 weight tiles (+ the up tiles
 //             for SwiGLU) and the matching bn x 64 activation tiles, 128-byte swizzled; weights
@@ -44,7 +43,6 @@ constexpr int kChunk = 16;
 constexpr int kMaxStages = 8;
 constexpr int kSmemLimit = 227 * 1024;
 constexpr uint32_t kABytes = kBM * kBK * 2;   // one 128 x 64 bf16 weight tile
-constexpr int kMaxTokList = 1024;             // token tiles a compacted launch can list
 
 struct TcArgs {
     CUtensorMap map_a, map_a2, map_b;   // weights, up weights (SwiGLU), activations
@@ -52,7 +50,6 @@ struct TcArgs {
     int bn, n_a, stages, n_bufs, tmem_cols;
     int pair;                  // 1: a unit is two adjacent 128-row tiles of one weight matrix
                                // (the second accumulator takes rows 128..255 of the pair)
-    int compact;               // EPI_KV_APPEND: skip the token tiles that hold no appended row
     int kbs;                   // 64-wide k-blocks per pipeline stage
     uint32_t b_bytes;          // bytes of one activation sub-tile (bn x 64 bf16)
     int evict_first;           // stream the weights with an L2 evict-first policy
@@ -84,7 +81,6 @@ __device__ __forceinline__ uint32_t atom_add_acq_rel(uint32_t* p, uint32_t v) {
 struct Geom {
     int n_units, n_tiles, tok_tiles, splits, kb_per_split, k_blocks, n_a, kbs, bn, n_bufs, pair;
     uint32_t b_bytes, stage_bytes, idesc;
-    const int* tok_list;       // token tiles in unit order (compacted launches), else nullptr
 };
 struct Unit {
     int group, n_tile, tok_tile, split, tile_id, kb0, kb1;
@@ -95,7 +91,6 @@ __device__ __forceinline__ Unit decode_unit(const Geom& a, int u) {
     x.tile_id = u / a.splits;
     int t = x.tile_id;
     x.tok_tile = t % a.tok_tiles;
-    if (a.tok_list) x.tok_tile = a.tok_list[x.tok_tile];
     t /= a.tok_tiles;
     x.n_tile = t % a.n_tiles;
     x.group = t / a.n_tiles;
@@ -145,7 +140,6 @@ __global__ void __launch_bounds__(kThreads, 1) gemm_tc_kernel(const __grid_const
     G.bn = args.bn;
     G.n_bufs = args.n_bufs;
     G.pair = args.pair;
-    G.tok_list = nullptr;
     G.b_bytes = args.b_bytes;
     G.stage_bytes = args.stage_bytes;
     G.idesc = args.idesc;
@@ -185,31 +179,6 @@ __global__ void __launch_bounds__(kThreads, 1) gemm_tc_kernel(const __grid_const
         asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
         asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
     }
-    // Compacted launch (a context fill of sequences with different lengths, token row
-    // b * n_max + r): after the dependency wait, warp 0 lists the token tiles that hold at least
-    // one appended row (r < app_cnt[b]); units then run over the listed tiles only.
-    int* const tok_list = reinterpret_cast<int*>(misc + 4);
-    if (args.compact) {
-        pdl_wait();
-        if (tst && threadIdx.x == 0) atomicMin(tst + args.t_slots, (unsigned long long)globaltimer_ns());
-        if (warp == 0) {
-            const int nm = args.ep.n_max;
-            int cnt = 0;
-            for (int base = 0; base < args.tok_tiles; base += 32) {
-                const int tt = base + lane;
-                bool v = false;
-                if (tt < args.tok_tiles) {
-                    const int r0 = tt * G.bn, r1 = min(args.ep.m_tok, r0 + G.bn);
-                    for (int b = r0 / nm; b <= (r1 - 1) / nm && !v; ++b)
-                        v = args.ep.app_cnt[b] > max(0, r0 - b * nm);
-                }
-                const unsigned m = __ballot_sync(0xffffffffu, v);
-                if (v) tok_list[cnt + __popc(m & ((1u << lane) - 1u))] = tt;
-                cnt += __popc(m);
-            }
-            if (lane == 0) misc[3] = (uint32_t)cnt;
-        }
-    }
     if (warp == 5) {
         asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(
                          smem_u32(&misc[0])),
@@ -222,11 +191,6 @@ __global__ void __launch_bounds__(kThreads, 1) gemm_tc_kernel(const __grid_const
     tc_fence_after();
     const uint32_t tmem = misc[0];
     volatile int* abort_flag = reinterpret_cast<volatile int*>(&misc[1]);
-    if (args.compact) {
-        G.n_units = args.n_units / args.tok_tiles * (int)misc[3];
-        G.tok_tiles = (int)misc[3];
-        G.tok_list = tok_list;
-    }
     const int acc_cols = G.n_a * G.bn;
 
     if (warp == 4) {
@@ -251,7 +215,7 @@ __global__ void __launch_bounds__(kThreads, 1) gemm_tc_kernel(const __grid_const
             int pend_kx[kMaxStages], pend_nk[kMaxStages], pend_tok[kMaxStages], pend_grp[kMaxStages];
             uint32_t pend_st[kMaxStages];
             int npend = 0;
-            bool waited = args.compact != 0;   // a compacted launch waited before the unit list
+            bool waited = false;
             auto load_b = [&](uint32_t st, int kx0, int nk, int tok_tile, int group, uint32_t bar) {
                 if constexpr (kAux) {
                     for (int j = 0; j < nk; ++j) {
@@ -698,10 +662,7 @@ cudaError_t launch_gemm_tc(dflare_ctx* c, const GemmDesc& g, cudaStream_t s, std
     // (512 contiguous bytes of every weight row; 128-byte rows per request leave DRAM bandwidth
     // unused), fewer when two stages do not fit.
     const int epi_bytes = a.n_a * kChunk * 128 * 4;
-    // a context fill over several token tiles lists the tiles that hold appended rows (the
-    // sequences of one call can have very different lengths: rows past app_cnt are padding)
-    a.compact = (g.ep.kind == EPI_KV_APPEND && a.tok_tiles > 1 && a.tok_tiles <= kMaxTokList) ? 1 : 0;
-    const int misc_bytes = 16 + (a.compact ? 4 * kMaxTokList : 0);
+    const int misc_bytes = 16;
     const int fixed = 1024 + epi_bytes + 8 * (2 * kMaxStages + 5) + misc_bytes;
     const int budget = g.max_smem > 0 ? std::min(g.max_smem, kSmemLimit) : kSmemLimit;
     if (g.kbs > 0) {

@@ -240,6 +240,9 @@ bool encode_tma_bf16(CUtensorMap* m, const void* base, int rank, const uint64_t*
 // the same over fp32 elements
 bool encode_tma_f32(CUtensorMap* m, const void* base, int rank, const uint64_t* dims,
                     const uint64_t* strides_bytes, const uint32_t* box);
+// the two-SM GEMM for many token rows: whether it takes the projection, and its launch
+bool gemm_pair_fits(const dflare_ctx* c, const GemmDesc& g);
+cudaError_t launch_gemm_pair(dflare_ctx* c, const GemmDesc& g, cudaStream_t s, std::string* why);
 cudaError_t launch_gemm_simt(dflare_ctx* c, const GemmDesc& g, cudaStream_t s);
 cudaError_t launch_fusion_alpha(dflare_ctx* c, cudaStream_t s);
 cudaError_t launch_fuse_begin(dflare_ctx* c, const int32_t* n_new, int n_max, cudaStream_t s);

@@ -18,17 +18,21 @@ def _shape(**kw):
     return synth.Shape(**base)
 
 
-def _step_matches_oracle(w, flags=0):
+def _step_matches_oracle(w, flags=0, **variant):
     """A fill of w.ctx_lens in one call, every cached key and value, and one drafted block."""
-    g = GpuSide(w, flags=flags)
-    o = oracle_for(w, g.W)
+    W = dict(synth.weights(w))
+    if variant:
+        W.update(synth.variant_weights(w))
+    g = GpuSide(w, flags=flags, weights=W)
+    o = oracle_for(w, W, **variant)
     got = f64(g.fuse(w.ctx_lens))
     for b, n in enumerate(w.ctx_lens):
         F = o.fuse_context(b, synth.hidden_states(w, b, 0, n))
         for i in range(w.shape.n_draft_layers):
-            check_rows(w, got[i, b, :n], F[i], f"F seq {b} layer {i}")
+            slot = 0 if variant.get("dflash_fc") else i
+            check_rows(w, got[slot, b, :n], F[slot], f"F seq {b} layer {i}")
             k, v = g.lib.read_kv(i, b, 0, n)
-            check_kv(w, o, f64(k), f64(v), got[i, b, :n], np.arange(n), i, f"seq {b} layer {i}")
+            check_kv(w, o, f64(k), f64(v), got[slot, b, :n], np.arange(n), i, f"seq {b} layer {i}")
     x_t = synth.initial_tokens(w)
     tok, logits, hidden = g.draft(x_t)
     for b in range(w.batch):
@@ -60,6 +64,36 @@ def test_simt_gemm_on_bf16_matches_oracle():
     """The CUDA-core GEMM on bf16 weights (a cross-check of the tensor-core GEMM)."""
     from paper_2606_02091_gb300 import FLAG_SIMT_GEMM
     _step_matches_oracle(synth.Workload("simt_bf16", _shape(d=320, ffn=192, vocab=333, block=9), (40, 3), 0.8, 35), FLAG_SIMT_GEMM)
+
+
+# bf16 projections of more than 128 token rows (two-SM tiles of 256 rows x 64 to 256 features): one row
+# past 128 (gate/up only) with a vocabulary that no 16-byte row fits, one past the 176 of the summed
+# projections, a second 256-row tile of one row, odd counts of 64-wide k-blocks (5, 3, 17), feature
+# counts that end inside a tile, both head sizes, and fills whose token tiles are partly or all padding
+PAIR_CASES = [
+    synth.Workload("pair_129", _shape(block=3, vocab=1003, ffn=192, d=320), tuple(3 + b % 5 for b in range(43)), 0.8, 41),
+    synth.Workload("pair_192", _shape(block=32, vocab=1000, ffn=1088, d=320, n_q_heads=8), (40, 3, 33, 1, 17, 64), 0.8, 42),
+    synth.Workload("pair_fill_257", _shape(head_dim=128, ffn=192), (257,), 0.8, 43),
+    synth.Workload("pair_288", _shape(block=32, vocab=2004, head_dim=128, ffn=704, d=576), (300, 1, 2, 5, 257, 9, 3, 30, 64), 0.8, 44),
+]
+
+
+@pytest.mark.parametrize("w", PAIR_CASES, ids=lambda w: w.name)
+@pytest.mark.parametrize("flag", ["", "FLAG_DETERMINISTIC"])
+def test_two_sm_gemm_matches_oracle(w, flag):
+    import paper_2606_02091_gb300 as P
+    _step_matches_oracle(w, getattr(P, flag) if flag else 0)
+
+
+@pytest.mark.parametrize("flag,kw", [("FLAG_FUSION_FC", dict(fusion_fc=True)), ("FLAG_DFLASH_FC", dict(dflash_fc=True)),
+                                     ("FLAG_SHARED_KV", dict(shared_kv=True))], ids=lambda x: x if isinstance(x, str) else "")
+@pytest.mark.parametrize("d", [256, 320])
+def test_two_sm_gemm_of_the_variants_matches_oracle(flag, kw, d):
+    """Biased and grouped stores, a contraction across stacked token groups (4 and 5 k-blocks each),
+    token groups shared by all weight groups, weight groups with rows between them."""
+    import paper_2606_02091_gb300 as P
+    w = synth.Workload("pair_variant", _shape(d=d, n_target_layers=3), (150, 90), 0.8, 45)
+    _step_matches_oracle(w, getattr(P, flag), **kw)
 
 
 @pytest.mark.parametrize("vocab,block,sampled", [(1000, 8, False), (1003, 8, False), (1000, 8, True), (1003, 5, True), (300, 1, False)])
