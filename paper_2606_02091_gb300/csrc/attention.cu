@@ -29,6 +29,7 @@
 
 #include "common.cuh"
 #include "internal.h"
+#include "umma.cuh"
 
 namespace cg = cooperative_groups;
 
@@ -770,6 +771,7 @@ __global__ void __launch_bounds__(kTThreads, 1) attn_tc_kernel(const __grid_cons
     const int s = (int)cluster.block_rank();
     const int g = blockIdx.y % a.hkv, qt = blockIdx.y / a.hkv, b = blockIdx.z;
     const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
+    const bool leader = elect_one();   // the thread that issues a producer or MMA warp's work
     const int R = a.B * a.G;
     const int rows = min(kTQ, R - qt * kTQ);    // query rows of this tile
 
@@ -844,9 +846,9 @@ __global__ void __launch_bounds__(kTThreads, 1) attn_tc_kernel(const __grid_cons
                 tma_tile(dst, v ? &maps.vd : &maps.kd, h * 64, b * a.B, g, bar);
         }
     };
-    int issued = 0;   // warps 8 (K) and 9 (V), lane 0
+    int issued = 0;   // warps 8 (K) and 9 (V), the leader
     // the first context tiles stream in while the projection drains; the block tile waits
-    if ((warp == 8 || warp == 9) && lane == 0)
+    if ((warp == 8 || warp == 9) && leader)
         for (; issued < min(NS, n_ct); ++issued) issue(issued, warp == 9);
     pdl_wait();
     if (a.t_stamps && tid == 0) atomicMin(a.t_stamps + a.t_slots, (unsigned long long)globaltimer_ns());
@@ -953,7 +955,7 @@ __global__ void __launch_bounds__(kTThreads, 1) attn_tc_kernel(const __grid_cons
     bool ok = true;
 
     if (warp == 8 || warp == 9) {
-        if (lane == 0) {
+        if (leader) {
             // ---------------- TMA producers, warp 8 for K and warp 9 for V: the slot of tile t is
             // refilled once the S (K) or the P V (V) of tile t - NS has completed
             const bool v = warp == 9;
@@ -973,7 +975,7 @@ __global__ void __launch_bounds__(kTThreads, 1) attn_tc_kernel(const __grid_cons
         }
         __syncwarp();
     } else if (warp == 10) {
-        if (lane == 0 && n_tiles > 0) {
+        if (leader && n_tiles > 0) {
             // ---------------- S issue (one thread): S of unit u into S buffer u % 2 once its K tiles
             // have landed and the softmax warps have read unit u - 2; descriptors advance by
             // address >> 4
@@ -1001,7 +1003,7 @@ __global__ void __launch_bounds__(kTThreads, 1) attn_tc_kernel(const __grid_cons
         }
         __syncwarp();
     } else if (warp == 11) {
-        if (lane == 0 && n_tiles > 0) {
+        if (leader && n_tiles > 0) {
             // ---------------- P V issue (one thread): O_q += P_t V_t once the V tile has landed and
             // group q = t & 1 has written P_t; the V slot is released when this P V completes
             const uint64_t dP = ta_desc_k(sbase + LY::P);
@@ -1123,7 +1125,7 @@ __global__ void __launch_bounds__(kTThreads, 1) attn_tc_kernel(const __grid_cons
         float2* xml = reinterpret_cast<float2*>(smem + LY::P + (uint32_t)q * (kTQ * 128));
         xml[row] = make_float2(n_tiles > q && ok ? m_used : -INFINITY, n_tiles > q && ok ? l : 0.f);
     }
-    if (!ok && lane == 0) atomicOr(a.err, DFLARE_DEVERR_TIMEOUT);
+    if (!ok) atomicOr(a.err, DFLARE_DEVERR_TIMEOUT);
     // every CTA of the cluster has finished with its stages (copies landed, MMAs drained) before
     // any partial is pushed into them
     __syncthreads();
