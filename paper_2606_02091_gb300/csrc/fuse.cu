@@ -9,11 +9,13 @@
 #include <math.h>
 
 #include <algorithm>
+#include <type_traits>
 
 #include <cooperative_groups.h>
 
 #include "common.cuh"
 #include "internal.h"
+#include "umma.cuh"
 
 namespace cg = cooperative_groups;
 
@@ -184,18 +186,25 @@ __global__ void __launch_bounds__(256) fuse_layers_kernel(
 }
 
 // Many positions (context fill): a persistent grid of one or two CTAs per SM walks the positions
-// (no cluster). Warp-specialised: the last warp's first thread streams the T target rows of each
-// position (d contiguous elements each) through a ring of `ns` shared-memory stages of kRB rows as
-// 1-D bulk copies, the stage sequence running on across positions; the other warps (one thread
-// per 8 features) consume the stages. Each stage has a "full" mbarrier (the copies landed) and an
-// "empty" one that every consumer warp arrives on once it has read the stage, which is what the
-// producer waits for before refilling it: no CTA barrier per stage, and up to ns - 1 stages in
-// flight while one is summed. Thread t forms the D (<= DMAX) draft-layer sums of features
-// [8t, 8t + 8) in registers; at the end of a position the consumer warps reduce the D sums of
-// squares (warp shuffles, then the warps' partials in order) behind a named barrier. Every wait
-// is bounded; a CTA that times out sets DFLARE_DEVERR_TIMEOUT and stops.
-constexpr int kRB = 4;          // target rows per stage
+// (no cluster). The T target rows of each position (d contiguous elements each) stream through a ring of
+// `ns` shared-memory stages of kRB rows as 1-D bulk copies, the stage sequence running on across
+// positions. Each stage has a "full" mbarrier (the copies landed) and an "empty" one that every warp
+// arrives on once it has read the stage; the warps take turns at refilling a slot, so no warp exists only
+// to copy: with one, an SM sub-partition holds a warp more and every thread a fifth fewer registers, and
+// the 128 sums of eight draft layers did not fit. Thread t forms the D (<= DMAX) draft-layer sums of 8
+// features (D <= 5) or two groups of 8 (more: half the reads of the weights alpha per sum, which at one
+// group cost as many shared-memory clocks as the rows) in registers; at the end of a position the D sums
+// of squares take 9 shuffles and one named barrier. Every wait is bounded; a CTA that times out sets
+// DFLARE_DEVERR_TIMEOUT and stops.
+// Bound by HBM for up to four draft layers, by the fp32 FMAs above (10.4k of 20k clocks a position at D 8,
+// d 4096). Measured, target rows read + fused rows written per second against a producer warp, one group
+// and three barriers a position: d 4096 D 8 4.0 -> 4.8 TB/s, D 4 5.5 -> 6.3, D 2 5.5 -> 6.2; d 2560 D 5
+// (2048 positions) 4.3 -> 4.7. Stages of 3 / 4 / 6 / 9 rows at D 8: 679 / 652 / 631 / 827 us for 8192 positions;
+// refilling one stage behind instead of two 631 -> 615.
+constexpr int kLag = 1;         // stages between a slot's use and its refill
 constexpr int kMaxNS = 16;      // most stages in the ring
+constexpr int kMinNS = 3;
+constexpr size_t kRingBytes = 200 * 1024;
 constexpr uint64_t kFillWaitNs = 2000000000ull;
 
 __device__ __forceinline__ bool fill_try(uint32_t bar, uint32_t parity) {
@@ -258,22 +267,25 @@ __device__ __forceinline__ void load8x2(const float* p, f32x2* h) {
     h[3] = pk2(b.z, b.w);
 }
 
-template <class T, int DMAX>
+template <class T>
+constexpr int kRowsPerStage = sizeof(T) == 2 ? 6 : 3;   // target rows
+
+template <class T, int DMAX, int NF>
 __device__ __forceinline__ void fuse_rows_body(
     const T* __restrict__ H, const float* __restrict__ alpha, const T* __restrict__ gain,
     T* __restrict__ F, T* __restrict__ F_out, const int32_t* __restrict__ app_cnt, int D, int Tn,
     int batch, int n_max, int d, long long f_layer_rows, float eps, int ns, uint32_t* err) {
+    constexpr int kRB = kRowsPerStage<T>;
     pdl_trigger();
     extern __shared__ __align__(128) uint8_t stage_mem[];   // [ns][kRB][d]
     constexpr int DP = (DMAX + 1) & ~1;                       // DMAX rounded up to even
     __shared__ __align__(16) f32x2 s_alpha[64 * DP];          // [j][i] = (alpha_ij, alpha_ij), Tn <= 64
-    __shared__ float red[16][DMAX];
-    __shared__ float inv_s[DMAX];
+    __shared__ float red[2][16][8];       // the warps' sums of squares, by parity of the position
+    __shared__ int s_cnt[64];             // appended rows per sequence
     __shared__ __align__(8) uint64_t full_bar[kMaxNS], empty_bar[kMaxNS];
     __shared__ int abort_flag;
     const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
-    const int n_cw = (int)(blockDim.x >> 5) - 1;   // consumer warps; the last warp produces
-    const int n_ct = n_cw * 32;
+    const int n_cw = (int)(blockDim.x >> 5), n_ct = (int)blockDim.x;
     const uint32_t fb0 = (uint32_t)__cvta_generic_to_shared(&full_bar[0]);
     const uint32_t eb0 = (uint32_t)__cvta_generic_to_shared(&empty_bar[0]);
     const uint32_t sbase = (uint32_t)__cvta_generic_to_shared(stage_mem);
@@ -291,6 +303,7 @@ __device__ __forceinline__ void fuse_rows_body(
         const float a = i < D ? alpha[i * Tn + j] : 0.f;
         s_alpha[k] = pk2(a, a);
     }
+    for (int k = tid; k < batch; k += blockDim.x) s_cnt[k] = app_cnt[k];
     __syncthreads();
     volatile int* abrt = &abort_flag;
     const int n_pos = batch * n_max;
@@ -298,7 +311,7 @@ __device__ __forceinline__ void fuse_rows_body(
     const uint32_t row_bytes = (uint32_t)(d * sizeof(T));
     const int nst = (Tn + kRB - 1) / kRB;   // stages per position
     // this CTA's positions pid = blockIdx.x + k * gridDim.x that have rows to append
-    auto valid = [&](int pid) { return pid % n_max < app_cnt[pid / n_max]; };
+    auto valid = [&](int pid) { return pid % n_max < s_cnt[pid / n_max]; };
     auto next_pos = [&](int pid) {
         for (pid += gridDim.x; pid < n_pos; pid += gridDim.x)
             if (valid(pid)) return pid;
@@ -307,117 +320,203 @@ __device__ __forceinline__ void fuse_rows_body(
     int first = (int)blockIdx.x;
     if (first < n_pos && !valid(first)) first = next_pos(first);
 
-    if (warp == n_cw) {
-        // ---------------- producer: one thread streams every stage of every position in turn
-        if (lane == 0) {
-            int g = 0;
-            bool ok = true;
-            for (int pid = first; pid < n_pos && ok; pid = next_pos(pid)) {
-                for (int k = 0; k < nst; ++k, ++g) {
-                    const int st = g % ns, use = g / ns;
-                    if (use > 0 && !fill_wait(eb0 + 8u * st, (uint32_t)((use - 1) & 1), abrt)) {
-                        ok = false;
-                        break;
-                    }
-                    const int j0 = k * kRB, nr = min(kRB, Tn - j0);
-                    asm volatile("mbarrier.arrive.expect_tx.shared::cta.b64 _, [%0], %1;" ::"r"(fb0 + 8u * st),
-                                 "r"((uint32_t)nr * row_bytes)
-                                 : "memory");
-                    for (int u = 0; u < nr; ++u)
-                        asm volatile(
-                            "cp.async.bulk.shared::cluster.global.mbarrier::complete_tx::bytes [%0], [%1], %2, [%3];" ::"r"(
-                                sbase + (uint32_t)(st * kRB + u) * row_bytes),
-                            "l"(H + (size_t)(j0 + u) * lstride + (size_t)pid * d), "r"(row_bytes),
-                            "r"(fb0 + 8u * st)
-                            : "memory");
+    // The stages run on across positions. Stage g goes into slot g % ns; the ring is filled once at the
+    // start, then each step's refill is issued by one elected thread, warp g % n_cw at its step g, into
+    // the slot of stage g - kLag, which the other warps have left by then as a rule. (ppid, pk): the
+    // next stage to issue, tracked by every thread.
+    int ppid = first, pk = 0;
+    auto next_stage = [&] {
+        if (++pk == nst) {
+            pk = 0;
+            ppid = next_pos(ppid);
+        }
+    };
+    auto issue = [&](int slot) {
+        const int j0 = pk * kRB, nr = min(kRB, Tn - j0);
+        const uint32_t bar = fb0 + 8u * slot;
+        asm volatile("mbarrier.arrive.expect_tx.shared::cta.b64 _, [%0], %1;" ::"r"(bar), "r"((uint32_t)nr * row_bytes)
+                     : "memory");
+        for (int u = 0; u < nr; ++u)
+            asm volatile(
+                "cp.async.bulk.shared::cluster.global.mbarrier::complete_tx::bytes [%0], [%1], %2, [%3];" ::"r"(
+                    sbase + (uint32_t)(slot * kRB + u) * row_bytes),
+                "l"(H + (size_t)(j0 + u) * lstride + (size_t)ppid * d), "r"(row_bytes), "r"(bar)
+                : "memory");
+    };
+    for (int i = 0; i < ns && ppid < n_pos; ++i, next_stage())
+        if (warp == 0 && elect_one()) issue(i);
+
+    {
+        // thread t owns NF groups of 8 features, n_ct groups apart; a thread without its last group reads
+        // group 0 instead and drops the result
+        int e[NF], er[NF];
+#pragma unroll
+        for (int c = 0; c < NF; ++c) {
+            e[c] = (tid + c * n_ct) * 8;
+            er[c] = e[c] < d ? e[c] : 0;
+        }
+        const T* stg = reinterpret_cast<const T*>(stage_mem);
+        int st = 0, par = 0, turn = 0;         // slot; parity of the position; warp that refills
+        int rst = -kLag;                       // slot to refill (negative: none yet)
+        uint32_t phase = 0, rphase = 0;
+        bool ok = true;
+        f32x2 acc2[DMAX][4 * NF];
+        // one target row, in G of the NF groups: a warp whose last group lies past d leaves it out
+        const bool all_groups = NF == 1 || (warp * 32 + (NF - 1) * n_ct) * 8 < d;
+        auto add_row = [&](auto groups, const T* row, int j) {
+            constexpr int G = decltype(groups)::value;
+            f32x2 h[4 * G];
+#pragma unroll
+            for (int c = 0; c < G; ++c) load8x2(row + er[c], h + 4 * c);
+#pragma unroll
+            for (int i = 0; i < DP; i += 2) {
+                const uint4 a4 = *reinterpret_cast<const uint4*>(&s_alpha[j * DP + i]);
+                const f32x2 a0 = ((f32x2)a4.y << 32) | a4.x, a1 = ((f32x2)a4.w << 32) | a4.z;
+#pragma unroll
+                for (int q = 0; q < 4 * G; ++q) acc2[i][q] = fma2(a0, h[q], acc2[i][q]);
+                if (i + 1 < DMAX) {
+                    const int i1 = i + 1 < DMAX ? i + 1 : i;
+#pragma unroll
+                    for (int q = 0; q < 4 * G; ++q) acc2[i1][q] = fma2(a1, h[q], acc2[i1][q]);
                 }
             }
-            // after a timeout: every issued copy lands before the CTA exits (bounded again)
-            if (!ok || *abrt) {
-                volatile int never = 0;
-                for (int q = max(0, g - ns); q < g; ++q)
-                    fill_wait(fb0 + 8u * (q % ns), (uint32_t)((q / ns) & 1), &never);
-                atomicOr(err, DFLARE_DEVERR_TIMEOUT);
-            }
-        }
-    } else {
-        // ---------------- consumers: thread t owns features [8t, 8t + 8)
-        const int e0 = tid * 8;
-        const bool act = e0 < d;
-        const T* stg = reinterpret_cast<const T*>(stage_mem);
-        int g = 0;
-        bool ok = true;
-        for (int pid = first; pid < n_pos && ok; pid = next_pos(pid)) {
+        };
+        for (int pid = first; pid < n_pos; pid = next_pos(pid)) {
             const int b = pid / n_max, r = pid % n_max;
-            f32x2 acc2[DMAX][4];
 #pragma unroll
             for (int i = 0; i < DMAX; ++i)
 #pragma unroll
-                for (int q = 0; q < 4; ++q) acc2[i][q] = 0ull;
-            for (int k = 0; k < nst; ++k, ++g) {
-                const int st = g % ns;
-                if (!fill_wait(fb0 + 8u * st, (uint32_t)((g / ns) & 1), abrt)) {
+                for (int q = 0; q < 4 * NF; ++q) acc2[i][q] = 0ull;
+            for (int k = 0; k < nst; ++k) {
+                if (!__all_sync(0xffffffffu, fill_wait(fb0 + 8u * st, phase, abrt))) {
                     ok = false;
                     break;
                 }
-                if (act) {
+                const T* row = stg + (size_t)st * kRB * d;
+                auto add_stage = [&](auto groups) {
+                    if ((k + 1) * kRB <= Tn) {   // no branch between the rows: their loads are in flight together
 #pragma unroll
-                    for (int u = 0; u < kRB; ++u) {
-                        const int j = k * kRB + u;
-                        if (j >= Tn) break;
-                        f32x2 h[4], a[DP];
-                        load8x2(stg + (size_t)(st * kRB + u) * d + e0, h);
-#pragma unroll
-                        for (int i = 0; i < DP; i += 2) {
-                            const uint4 a4 = *reinterpret_cast<const uint4*>(&s_alpha[j * DP + i]);
-                            a[i] = ((f32x2)a4.y << 32) | a4.x;
-                            a[i + 1] = ((f32x2)a4.w << 32) | a4.z;
-                        }
-#pragma unroll
-                        for (int i = 0; i < DMAX; ++i)
-#pragma unroll
-                            for (int q = 0; q < 4; ++q) acc2[i][q] = fma2(a[i], h[q], acc2[i][q]);
+                        for (int u = 0; u < kRB; ++u) add_row(groups, row + u * d, k * kRB + u);
+                    } else {
+                        for (int j = k * kRB; j < Tn; ++j, row += d) add_row(groups, row, j);
                     }
-                }
+                };
+                if (all_groups)
+                    add_stage(std::integral_constant<int, NF>{});
+                else if constexpr (NF > 1)
+                    add_stage(std::integral_constant<int, NF - 1>{});
                 __syncwarp();
                 if (lane == 0) asm volatile("mbarrier.arrive.shared::cta.b64 _, [%0];" ::"r"(eb0 + 8u * st) : "memory");
+                if (rst >= 0 && ppid < n_pos) {
+                    if (warp == turn && elect_one()) {
+                        if (fill_wait(eb0 + 8u * rst, rphase, abrt))
+                            issue(rst);
+                        else
+                            ok = false;
+                    }
+                    next_stage();
+                }
+                if (++turn == n_cw) turn = 0;
+                if (++rst == ns) {
+                    rst = 0;
+                    rphase ^= 1u;
+                }
+                if (++st == ns) {
+                    st = 0;
+                    phase ^= 1u;
+                }
             }
-            // the consumer warps leave the position loop together: a warp whose wait ran out sets
-            // the abort flag, which every other consumer sees at the barrier below
-            asm volatile("bar.sync 1, %0;" ::"r"(n_ct) : "memory");
-            if (!ok || *abrt) break;
-            float acc[DMAX][8];
+            // the first gains of bf16 rows arrive behind the reduction, the others kGP layers ahead
+            constexpr int kGP = DMAX < 4 ? DMAX : 4;
+            uint4 graw[kGP][NF];
+            auto fetch_gain = [&](int i) {
+                if constexpr (sizeof(T) == 2) {
+                    if (i < D) {
 #pragma unroll
-            for (int i = 0; i < DMAX; ++i)
+                        for (int c = 0; c < NF; ++c)
+                            graw[i % kGP][c] = __ldg(reinterpret_cast<const uint4*>(gain + (size_t)i * d + er[c]));
+                    }
+                }
+            };
 #pragma unroll
-                for (int q = 0; q < 4; ++q) upk2(acc2[i][q], acc[i][2 * q], acc[i][2 * q + 1]);
+            for (int i = 0; i < kGP; ++i) fetch_gain(i);
+            // sums of squares: eight values over 32 lanes by halving exchanges (9 shuffles; lane holds
+            // value lane / 4 at the end), the warps' sums through shared memory
+            float v[8];
+#pragma unroll
+            for (int i = 0; i < 8; ++i) v[i] = 0.f;
 #pragma unroll
             for (int i = 0; i < DMAX; ++i) {
-                float v = 0.f;
 #pragma unroll
-                for (int e = 0; e < 8; ++e) v = fmaf(acc[i][e], acc[i][e], v);
-                v = warp_sum(v);
-                if (lane == 0) red[warp][i] = v;
-            }
-            asm volatile("bar.sync 1, %0;" ::"r"(n_ct) : "memory");
-            if (tid < D) {
-                float tot = 0.f;
-                for (int w = 0; w < n_cw; ++w) tot += red[w][tid];
-                inv_s[tid] = inv_rms(tot, d, eps);
-            }
-            asm volatile("bar.sync 1, %0;" ::"r"(n_ct) : "memory");
-            if (act) {
+                for (int c = 0; c < NF; ++c) {
+                    f32x2 s2 = 0ull;
 #pragma unroll
-                for (int i = 0; i < DMAX; ++i) {
-                    if (i >= D) break;
-                    float gg[8], o[8];
-                    load8(gain + (size_t)i * d + e0, gg);
-                    const float inv = inv_s[i];
-#pragma unroll
-                    for (int e = 0; e < 8; ++e) o[e] = gg[e] * (acc[i][e] * inv);
-                    store8(F + ((size_t)i * f_layer_rows + pid) * d + e0, o);
-                    if (F_out) store8(F_out + (((size_t)i * batch + b) * n_max + r) * d + e0, o);
+                    for (int q = 0; q < 4; ++q) s2 = fma2(acc2[i][4 * c + q], acc2[i][4 * c + q], s2);
+                    float lo, hi;
+                    upk2(s2, lo, hi);
+                    if (e[c] < d) v[i] += lo + hi;
                 }
+            }
+#pragma unroll
+            for (int n = 4, o = 16; n > 0; n >>= 1, o >>= 1) {
+                const bool up = lane & o;
+#pragma unroll
+                for (int i = 0; i < n; ++i) {
+                    const float give = up ? v[i] : v[i + n], keep = up ? v[i + n] : v[i];
+                    v[i] = keep + __shfl_xor_sync(0xffffffffu, give, o);
+                }
+            }
+            v[0] += __shfl_xor_sync(0xffffffffu, v[0], 2);
+            v[0] += __shfl_xor_sync(0xffffffffu, v[0], 1);
+            if ((lane & 3) == 0) red[par][warp][lane >> 2] = v[0];
+            // one barrier a position: it also tells every consumer whether one of them timed out, so
+            // that they leave together
+            int bad;
+            asm volatile(
+                "{\n\t.reg .pred p, q;\n\t"
+                "setp.ne.s32 p, %1, 0;\n\t"
+                "barrier.cta.red.or.pred q, 1, %2, p;\n\t"
+                "selp.s32 %0, 1, 0, q;\n\t}"
+                : "=r"(bad)
+                : "r"(ok ? 0 : 1), "r"(n_ct)
+                : "memory");
+            if (bad) {   // its copies in flight land long before the millisecond is over
+                if (tid == 0) atomicOr(err, DFLARE_DEVERR_TIMEOUT);
+                const uint64_t t0 = globaltimer_ns();
+                while (globaltimer_ns() - t0 < 1000000ull) {
+                }
+                break;
+            }
+            // every warp adds the warps' sums itself: lane = value lane % 8, warps lane / 8, + 4, ...
+            float tot = 0.f;
+            for (int w = lane >> 3; w < n_cw; w += 4) tot += red[par][w][lane & 7];
+            tot += __shfl_xor_sync(0xffffffffu, tot, 8);
+            tot += __shfl_xor_sync(0xffffffffu, tot, 16);
+            const float inv_l = inv_rms(tot, d, eps);
+            par ^= 1;
+#pragma unroll
+            for (int i = 0; i < DMAX; ++i) {
+                if (i >= D) break;
+                const float inv = __shfl_sync(0xffffffffu, inv_l, i);
+#pragma unroll
+                for (int c = 0; c < NF; ++c) {
+                    if (e[c] >= d) continue;
+                    float gg[8], o[8];
+                    if constexpr (sizeof(T) == 2)
+                        load8(reinterpret_cast<const T*>(&graw[i % kGP][c]), gg);
+                    else
+                        load8(gain + (size_t)i * d + e[c], gg);
+#pragma unroll
+                    for (int q = 0; q < 4; ++q) {
+                        float lo, hi;
+                        upk2(acc2[i][4 * c + q], lo, hi);
+                        o[2 * q] = gg[2 * q] * (lo * inv);
+                        o[2 * q + 1] = gg[2 * q + 1] * (hi * inv);
+                    }
+                    store8(F + ((size_t)i * f_layer_rows + pid) * d + e[c], o);
+                    if (F_out) store8(F_out + (((size_t)i * batch + b) * n_max + r) * d + e[c], o);
+                }
+                if (i + kGP < DMAX) fetch_gain(i + kGP);
             }
         }
     }
@@ -429,15 +528,13 @@ __device__ __forceinline__ void fuse_rows_body(
         T *__restrict__ F, T *__restrict__ F_out, const int32_t *__restrict__ app_cnt, int D,         \
         int Tn, int batch, int n_max, int d, long long f_layer_rows, float eps, int ns, uint32_t *err
 #define FUSE_ROWS_ARGS H, alpha, gain, F, F_out, app_cnt, D, Tn, batch, n_max, d, f_layer_rows, eps, ns, err
-// one CTA per SM (up to 512 consumer threads), or two per SM for d <= 2560 and D <= 5 (registers
-// capped; eight sums of eight features do not fit without spills)
-template <class T, int DMAX>
-__global__ void __launch_bounds__(544, 1) fuse_rows_kernel(FUSE_ROWS_PARAMS) {
-    fuse_rows_body<T, DMAX>(FUSE_ROWS_ARGS);
+template <class T, int DMAX, int NF>
+__global__ void __launch_bounds__(512 / NF, 1) fuse_rows_kernel(FUSE_ROWS_PARAMS) {
+    fuse_rows_body<T, DMAX, NF>(FUSE_ROWS_ARGS);
 }
 template <class T, int DMAX>
-__global__ void __launch_bounds__(352, 2) fuse_rows2_kernel(FUSE_ROWS_PARAMS) {
-    fuse_rows_body<T, DMAX>(FUSE_ROWS_ARGS);
+__global__ void __launch_bounds__(320, 2) fuse_rows2_kernel(FUSE_ROWS_PARAMS) {
+    fuse_rows_body<T, DMAX, 1>(FUSE_ROWS_ARGS);
 }
 #undef FUSE_ROWS_PARAMS
 #undef FUSE_ROWS_ARGS
@@ -456,30 +553,27 @@ cudaError_t fuse_layers_t(dflare_ctx* c, const void* hidden, int n_max, void* fu
     // context fill: warp-specialised CTAs of d / 8 consumer threads and a producer warp, two per SM
     // when their registers allow (rings of about 100 KB), else one (about 200 KB); at most kMaxNS
     // stages of kRB rows
-    const int cthreads = ((g.d / 8 + 31) / 32) * 32;
-    const size_t stage_bytes = (size_t)kRB * g.d * sizeof(T);
-    if ((long long)c->batch * n_max >= 2LL * c->num_sms && cthreads <= 512 && g.n_draft_layers <= 8 &&
-        g.n_target_layers <= 64 && 3 * stage_bytes <= 200 * 1024) {
-        const int threads = cthreads + 32;
+    const size_t stage_bytes = (size_t)kRowsPerStage<T> * g.d * sizeof(T);
+    const int Dn = g.n_draft_layers, nf = Dn <= 5 ? 1 : 2;
+    const int threads = std::min(512 / nf, (g.d / 8 + 31) / 32 * 32);   // (d <= 4096)
+    if ((long long)c->batch * n_max >= 2LL * c->num_sms && Dn <= 8 && g.n_target_layers <= 64 &&
+        kMinNS * stage_bytes <= kRingBytes) {
         static PerDeviceOnce rconf;
         const cudaError_t re = rconf([] {
-            for (auto k : {fuse_rows_kernel<T, 4>, fuse_rows_kernel<T, 5>, fuse_rows_kernel<T, 8>,
-                           fuse_rows2_kernel<T, 4>, fuse_rows2_kernel<T, 5>, fuse_rows2_kernel<T, 8>}) {
-                cudaError_t e = cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                                     200 * 1024);
+            for (auto k : {fuse_rows_kernel<T, 4, 1>, fuse_rows_kernel<T, 5, 1>, fuse_rows_kernel<T, 8, 2>,
+                           fuse_rows2_kernel<T, 4>, fuse_rows2_kernel<T, 5>}) {
+                cudaError_t e = cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kRingBytes);
                 if (e != cudaSuccess) return e;
             }
             return cudaSuccess;
         });
         if (re != cudaSuccess) return re;
-        const int Dn = g.n_draft_layers;
-        auto rk1 = Dn <= 4 ? fuse_rows_kernel<T, 4> : Dn == 5 ? fuse_rows_kernel<T, 5> : fuse_rows_kernel<T, 8>;
-        auto rk2 = Dn <= 4 ? fuse_rows2_kernel<T, 4> : Dn == 5 ? fuse_rows2_kernel<T, 5> : fuse_rows2_kernel<T, 8>;
-        auto rk = rk1;
-        int ns = (int)std::min<size_t>(kMaxNS, (200 * 1024) / stage_bytes), per_sm = 1;
-        const int ns2 = (int)std::min<size_t>(kMaxNS, (100 * 1024) / stage_bytes);
+        auto rk = Dn <= 4 ? fuse_rows_kernel<T, 4, 1> : Dn == 5 ? fuse_rows_kernel<T, 5, 1> : fuse_rows_kernel<T, 8, 2>;
+        auto rk2 = Dn <= 4 ? fuse_rows2_kernel<T, 4> : fuse_rows2_kernel<T, 5>;   // (D <= 5 below)
+        int ns = (int)std::min<size_t>(kMaxNS, kRingBytes / stage_bytes), per_sm = 1;
+        const int ns2 = (int)std::min<size_t>(kMaxNS, kRingBytes / 2 / stage_bytes);
         int fit = 0;
-        if (threads <= 352 && Dn <= 5 && ns2 >= 3 &&
+        if (threads <= 320 && Dn <= 5 && ns2 >= kMinNS &&
             cudaOccupancyMaxActiveBlocksPerMultiprocessor(&fit, rk2, threads, (size_t)ns2 * stage_bytes) ==
                 cudaSuccess && fit >= 2) {
             rk = rk2;

@@ -96,6 +96,23 @@ def test_two_sm_gemm_of_the_variants_matches_oracle(flag, kw, d):
     _step_matches_oracle(w, getattr(P, flag), **kw)
 
 
+# context fills of at least two positions per SM: one and two feature groups per thread (five and six draft
+# layers), two CTAs per SM, warps with and without their second group, target-layer counts that end inside
+# a stage of 6 (bf16) or 3 (fp32) rows, fewer target rows than a stage, positions past a sequence's end
+FILL_CASES = [
+    synth.Workload("fill_d2112_D6_T7", _shape(d=2112, n_draft_layers=6, n_target_layers=7, ffn=64, block=2), (170, 140), 0.8, 51),
+    synth.Workload("fill_d4096_D8_T3", _shape(d=4096, n_draft_layers=8, n_target_layers=3, ffn=64, block=2), (305,), 0.8, 52),
+    synth.Workload("fill_d704_D5_T13", _shape(d=704, n_draft_layers=5, n_target_layers=13, ffn=64, block=2), (300, 9), 0.8, 53),
+    synth.Workload("fill_d2816_D3_T6", _shape(d=2816, n_draft_layers=3, n_target_layers=6, ffn=64, block=2), (305,), 0.8, 54),
+    synth.Workload("fill_f32_d320_D7_T5", _shape(dtype="f32", d=320, n_draft_layers=7, n_target_layers=5, ffn=64, block=2), (306,), 0.8, 55),
+]
+
+
+@pytest.mark.parametrize("w", FILL_CASES, ids=lambda w: w.name)
+def test_fill_fusion_matches_oracle(w):
+    _step_matches_oracle(w)
+
+
 @pytest.mark.parametrize("vocab,block,sampled", [(1000, 8, False), (1003, 8, False), (1000, 8, True), (1003, 5, True), (300, 1, False)])
 def test_copies_to_aligned_and_unaligned_buffers_agree(vocab, block, sampled):
     """logits_out and hidden_out as written by the kernels (16-byte aligned buffers) and as copied
