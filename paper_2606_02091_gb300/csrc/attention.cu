@@ -613,18 +613,22 @@ struct TcAttnLayout {
     static constexpr bool PAIR = HD == 128;
     static constexpr int W = PAIR ? 2 : 1;                      // 64-key tiles per S unit
     static_assert(NS % 2 == 0, "pairs of adjacent K slots form one N 128 operand");
-    // After the key loop the (then idle) stages hold the cluster merge: the pushed partials O / l
-    // in fp16 [S RP <= 128 + 15 rows][HD], their (m, l) and the merge weights [RP][S].
+    // The cluster merge: the pushed partials O / l in fp16 [S RP rows][HD] and their (m, l). S RP is 128
+    // to 140 for 128 query rows; up to MD rows have a place of their own behind the barriers, more go
+    // into the stages once every CTA of the cluster is done with them. The merge weights [RP][16] lie in
+    // the P buffers, behind the groups' (m, l).
     static constexpr int MR = kTQ + kMaxSplits;
-    static constexpr uint32_t RO = 0;
-    static constexpr uint32_t RML = (uint32_t)MR * HD * 2;
-    static constexpr uint32_t RW = RML + (uint32_t)MR * 8;
+    static constexpr uint32_t MERGE = (BYTES + 15u) & ~15u;
+    static constexpr int MD = (int)((232448u - 1024u - MERGE) / (HD * 2 + 8));
+    static constexpr uint32_t RW = P + 2048;
+    static constexpr uint32_t TOTAL = MERGE + MD * (HD * 2 + 8);
     static constexpr uint32_t TMEM_COLS = 512;                  // S of two tile pairs (128 each), O_A, O_B
-    static_assert(RW + (uint32_t)MR * kMaxSplits * 4 <= NS * 2 * TB, "merge buffers exceed the stages");
-    static_assert(1024 + BYTES <= 232448, "tcgen05 attention exceeds 227 KB of shared memory");
+    static_assert((uint32_t)MR * (HD * 2 + 8) <= NS * 2 * TB, "merge buffers exceed the stages");
+    static_assert(2048 + (kTQ / 2) * kMaxSplits * 4 <= kTQ * 128, "merge weights exceed a P buffer");
+    static_assert(1024 + TOTAL <= 232448 && MD >= kTQ, "tcgen05 attention exceeds 227 KB of shared memory");
 };
 template <int HD>
-size_t tc_attn_smem_bytes() { return 1024 + TcAttnLayout<HD>::BYTES; }
+size_t tc_attn_smem_bytes() { return 1024 + TcAttnLayout<HD>::TOTAL; }
 
 __device__ __forceinline__ void ta_mbar_init(uint32_t bar, uint32_t count) {
     asm volatile("mbarrier.init.shared::cta.b64 [%0], %1;" ::"r"(bar), "r"(count) : "memory");
@@ -818,6 +822,8 @@ __global__ void __launch_bounds__(kTThreads, 1) attn_tc_kernel(const __grid_cons
     __syncthreads();
     ta_fence_after();
     const uint32_t tmem = misc[0];
+    // (waited for before the first store to another CTA's shared memory: by then it has started)
+    if (S > 1) asm volatile("barrier.cluster.arrive.release.aligned;" ::: "memory");
     // dependents are released only once this CTA holds its tensor memory, so a dependent CTA
     // that allocates before its own dependency wait can never hold columns this CTA waits for
     pdl_trigger();
@@ -1126,18 +1132,25 @@ __global__ void __launch_bounds__(kTThreads, 1) attn_tc_kernel(const __grid_cons
         xml[row] = make_float2(n_tiles > q && ok ? m_used : -INFINITY, n_tiles > q && ok ? l : 0.f);
     }
     if (!ok) atomicOr(a.err, DFLARE_DEVERR_TIMEOUT);
-    // every CTA of the cluster has finished with its stages (copies landed, MMAs drained) before
-    // any partial is pushed into them
     __syncthreads();
-    cluster.sync();
-    // Push the partial: both groups' (m, l, O) of query row r are combined and written to CTA
-    // r / RP at [s RP + r % RP]; warpgroup h (warps 4h .. 4h + 3, lane quarter = warp % 4) takes the
-    // head dims [h HD/2, h HD/2 + HD/2). A group without tiles (m = -inf) contributes nothing and
-    // its O is not read; the loads are guarded by warp votes, so they stay collective.
+    // Both groups' (m, l, O) of query row r are combined; warpgroup h (warps 4h .. 4h + 3, lane quarter =
+    // warp % 4) takes the head dims [h HD/2, h HD/2 + HD/2). One split: the row's result. Several: the
+    // partial goes to CTA r / RP at [s RP + r % RP] of its merge buffer; with more rows than that has,
+    // into its stages, once every CTA of the cluster has finished with its own (copies landed, MMAs
+    // drained). A group without tiles (m = -inf) contributes nothing and its O is not read; the loads are
+    // guarded by warp votes, so they stay collective.
     const int RP = (rows + S - 1) / S;
-    __half* rO = reinterpret_cast<__half*>(smem + LY::RO);
-    float2* rML = reinterpret_cast<float2*>(smem + LY::RML);
+    const bool own = S * RP <= LY::MD;
+    if (S > 1) asm volatile("barrier.cluster.wait.acquire.aligned;" ::: "memory");
+    if (!own && S > 1) cluster.sync();
+    __half* rO = reinterpret_cast<__half*>(smem + (own ? LY::MERGE : 0u));
+    float2* rML = reinterpret_cast<float2*>(smem + (own ? LY::MERGE + (uint32_t)LY::MD * HD * 2 : (uint32_t)LY::MR * HD * 2));
     float* rW = reinterpret_cast<float*>(smem + LY::RW);
+    // where row rr of the tile goes: block position rr / G, query head g G + rr % G
+    auto out_row = [&](int rr) {
+        const int rg = qt * kTQ + rr, kpos = rg / a.G, hh = rg - kpos * a.G;
+        return out + ((size_t)b * a.B + kpos) * a.d_q + (size_t)(g * a.G + hh) * HD;
+    };
     if (warp < 8 && (warp & 3) * 32 < rows) {
         const int r = tid & 127, half = warp >> 2;
         const bool row_ok = r < rows;
@@ -1150,26 +1163,24 @@ __global__ void __launch_bounds__(kTThreads, 1) attn_tc_kernel(const __grid_cons
         const float inv = lt > 0.f ? 1.0f / lt : 0.f;
         const float cA = wA * inv, cB = wB * inv;
         const int dst_cta = row_ok ? r / RP : 0, dst_row = s * RP + (row_ok ? r % RP : 0);
-        __half* dst = cluster.map_shared_rank(rO, dst_cta) + (size_t)dst_row * HD;
+        __half* dst = S > 1 ? cluster.map_shared_rank(rO, dst_cta) + (size_t)dst_row * HD : nullptr;
+        bf16* const orow = out_row(row_ok ? r : 0);
         const uint32_t lb = (uint32_t)((warp & 3) * 32) << 16;
         const bool anyA = __any_sync(0xffffffffu, hA), anyB = __any_sync(0xffffffffu, hB);
         if (anyA || anyB) {
 #pragma unroll
             for (int c = half * (HD / 64); c < (half + 1) * (HD / 64); ++c) {
-                float ov[32], ob[32];
-                if (anyA) {
-                    ta_ld32(tO(0) + lb + c * 32, ov);
-                } else {
-#pragma unroll
-                    for (int i = 0; i < 32; ++i) ov[i] = 0.f;
-                }
-                if (anyB) ta_ld32(tO(1) + lb + c * 32, ob);
+                uint32_t va[32], vb[32];
+                if (anyA) tmem_ld32_async(tO(0) + lb + c * 32, va);
+                if (anyB) tmem_ld32_async(tO(1) + lb + c * 32, vb);
+                tmem_wait_ld();
+                float ov[32];
 #pragma unroll
                 for (int i = 0; i < 32; ++i) {
-                    const float x = hA ? ov[i] * cA : 0.f;
-                    ov[i] = hB ? fmaf(ob[i], cB, x) : x;
+                    const float x = hA ? __uint_as_float(va[i]) * cA : 0.f;
+                    ov[i] = hB ? fmaf(__uint_as_float(vb[i]), cB, x) : x;
                 }
-                if (row_ok) {
+                if (row_ok && S > 1) {
 #pragma unroll
                     for (int k = 0; k < 4; ++k) {
                         uint4 u;
@@ -1178,44 +1189,46 @@ __global__ void __launch_bounds__(kTThreads, 1) attn_tc_kernel(const __grid_cons
                         for (int e = 0; e < 4; ++e) h[e] = __floats2half2_rn(ov[k * 8 + 2 * e], ov[k * 8 + 2 * e + 1]);
                         *reinterpret_cast<uint4*>(dst + c * 32 + k * 8) = u;
                     }
+                } else if (row_ok) {
+#pragma unroll
+                    for (int k = 0; k < 4; ++k) store8(orow + c * 32 + k * 8, ov + k * 8);
                 }
             }
         }
-        if (row_ok && half == 0)
+        if (row_ok && half == 0 && S > 1)
             *cluster.map_shared_rank(rML + dst_row, dst_cta) = make_float2(hA || hB ? M : -INFINITY, lt);
     }
-    // every partial has arrived; after this barrier no CTA touches another's shared memory
     ta_fence_before();
-    cluster.sync();
+    if (S > 1)   // every partial has arrived; after this barrier no CTA touches another's shared memory
+        cluster.sync();
+    else
+        __syncthreads();
     if (warp == 9) {
         ta_fence_after();
         asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(tmem), "r"(LY::TMEM_COLS)
                      : "memory");
     }
-    // merge this CTA's rows [s RP, min(rows, s RP + RP)): the weights of the S partials of each
-    // row (a partial with m = -inf weighs 0 and its O is not read), then 8 output elements per item
-    const int r0 = s * RP, nr = max(0, min(rows - r0, RP));
-    for (int i = tid; i < nr; i += kTThreads) {
-        float M = -INFINITY;
-        for (int p = 0; p < S; ++p) M = fmaxf(M, rML[p * RP + i].x);
-        float den = 0.f;
-        for (int p = 0; p < S; ++p) {
-            const float2 ml = rML[p * RP + i];
+    if (S > 1) {
+        // merge this CTA's rows [s RP, min(rows, s RP + RP)): a warp per row for the weights of its S
+        // partials (a partial with m = -inf weighs 0 and its O is not used), then 8 output elements per item
+        const int r0 = s * RP, nr = max(0, min(rows - r0, RP));
+        for (int i = warp; i < nr; i += kTThreads / 32) {
+            const float2 ml = lane < S ? rML[lane * RP + i] : make_float2(-INFINITY, 0.f);
+            const float M = warp_max(ml.x);
             const float w = ml.x == -INFINITY ? 0.f : ml.y * exp2f(ml.x - M);
-            rW[i * kMaxSplits + p] = w;
-            den += w;
+            const float den = warp_sum(w);
+            if (lane < S) rW[i * kMaxSplits + lane] = w * (1.0f / den);
         }
-        const float inv = 1.0f / den;
-        for (int p = 0; p < S; ++p) rW[i * kMaxSplits + p] *= inv;
-    }
-    __syncthreads();
-    for (int it = tid; it < nr * (HD / 8); it += kTThreads) {
-        const int i = it / (HD / 8), c = it % (HD / 8);
-        float acc[8] = {0.f, 0.f, 0.f, 0.f, 0.f, 0.f, 0.f, 0.f};
-        for (int p = 0; p < S; ++p) {
-            const float w = rW[i * kMaxSplits + p];
-            if (w != 0.f) {
-                const uint4 v = *reinterpret_cast<const uint4*>(rO + (size_t)(p * RP + i) * HD + c * 8);
+        __syncthreads();
+        for (int it = tid; it < nr * (HD / 8); it += kTThreads) {
+            const int i = it / (HD / 8), c = it % (HD / 8);
+            float acc[8] = {0.f, 0.f, 0.f, 0.f, 0.f, 0.f, 0.f, 0.f};
+            const __half* src = rO + (size_t)i * HD + c * 8;
+#pragma unroll 4
+            for (int p = 0; p < S; ++p) {
+                const float w = rW[i * kMaxSplits + p];
+                uint4 v = *reinterpret_cast<const uint4*>(src + (size_t)p * RP * HD);
+                if (w == 0.f) v = make_uint4(0u, 0u, 0u, 0u);
                 const __half2* hv = reinterpret_cast<const __half2*>(&v);
 #pragma unroll
                 for (int e = 0; e < 4; ++e) {
@@ -1224,9 +1237,8 @@ __global__ void __launch_bounds__(kTThreads, 1) attn_tc_kernel(const __grid_cons
                     acc[2 * e + 1] = fmaf(w, f.y, acc[2 * e + 1]);
                 }
             }
+            store8(out_row(r0 + i) + c * 8, acc);
         }
-        const int rg = qt * kTQ + r0 + i, kpos = rg / a.G, hh = rg % a.G;
-        store8(out + ((size_t)b * a.B + kpos) * a.d_q + (size_t)(g * a.G + hh) * HD + c * 8, acc);
     }
     if (a.t_stamps) {
         __syncthreads();
