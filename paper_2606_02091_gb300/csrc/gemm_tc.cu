@@ -45,7 +45,6 @@ constexpr int kBK = 64;
 constexpr int kChunk = 16;
 constexpr int kMaxStages = 8;
 constexpr int kSmemLimit = 227 * 1024;
-constexpr uint32_t kABytes = kBM * kBK * 2;   // one 128 x 64 bf16 weight tile
 
 // How a tile leaves the accumulators. OUT_REGS: chunks of 16 tokens turned token-major in shared memory
 // and finished by apply_epilogue. The others: every epilogue warp stages its 32 features of 16 or 32
@@ -63,6 +62,8 @@ struct TcArgs {
     CUtensorMap map_o;                  // output (out_mode != OUT_REGS)
     int n_units, n_tiles, tok_tiles, splits, kb_per_split, k_blocks;
     int bn, n_a, stages, n_bufs, tmem_cols;
+    int bm;                    // weight rows of a tile (128; fewer for SwiGLU: see launch_gemm_tc)
+    uint32_t a_bytes;          // bytes of one weight sub-tile (bm x 64 bf16)
     int pair;                  // 1: a unit is two adjacent 128-row tiles of one weight matrix
                                // (the second accumulator takes rows 128..255 of the pair)
     int kbs;                   // 64-wide k-blocks per pipeline stage
@@ -96,7 +97,7 @@ __device__ __forceinline__ uint32_t atom_add_acq_rel(uint32_t* p, uint32_t v) {
 // addressed for the tensor maps, so every asm with a memory clobber would otherwise reload them).
 struct Geom {
     int n_units, n_tiles, tok_tiles, splits, kb_per_split, k_blocks, n_a, kbs, bn, n_bufs, pair;
-    uint32_t b_bytes, stage_bytes, idesc;
+    uint32_t a_bytes, b_bytes, stage_bytes, idesc;
 };
 struct Unit {
     int group, n_tile, tok_tile, split, tile_id, kb0, kb1;
@@ -191,7 +192,7 @@ __device__ __forceinline__ void sum_partials(const float* part, const Geom& G, i
 }
 // A tile's results through this warp's staging slots and TMA (out_mode != OUT_REGS), CH tokens at a time:
 // lane = feature 32 warp + lane of the tile, so a token's 32 features are one conflict-free row of a slot
-// (128 bytes of fp32 in the copies' 128-byte swizzle, or 64 bytes of bf16).
+// (128 bytes of fp32 in the copies' 128-byte swizzle, or two boxes of 32 bytes of bf16).
 template <int CH>
 __device__ __forceinline__ void staged_out(const TcArgs& args, const Geom& G, const Unit& x, uint32_t taddr,
                                            const float* part, float* stage, int warp, int lane) {
@@ -199,7 +200,8 @@ __device__ __forceinline__ void staged_out(const TcArgs& args, const Geom& G, co
     const bool h16 = mode == OUT_SWIGLU;
     const uint32_t slot_bytes = CH * (h16 ? 64u : 128u);
     uint8_t* const base = reinterpret_cast<uint8_t*>(stage) + (uint32_t)(warp * args.n_slots) * slot_bytes;
-    const int n0 = x.n_tile * 128 + warp * 32;
+    const int n0 = x.n_tile * args.bm + warp * 32, nw = min(32, args.bm - warp * 32);   // features of this warp
+    if (nw <= 0) return;
     int slot = 0;
     for (int c0 = 0; c0 < bn; c0 += CH) {
         uint32_t v[CH], up[CH];
@@ -227,7 +229,7 @@ __device__ __forceinline__ void staged_out(const TcArgs& args, const Geom& G, co
         if (h16) {
 #pragma unroll
             for (int c = 0; c < CH; ++c)
-                *reinterpret_cast<bf16*>(sl + c * 64 + lane * 2) =
+                *reinterpret_cast<bf16*>(sl + (lane >> 4) * (CH * 32) + c * 32 + (lane & 15) * 2) =
                     from_f<bf16>(silu_f(__uint_as_float(v[c])) * __uint_as_float(up[c]));
         } else {
 #pragma unroll
@@ -238,10 +240,14 @@ __device__ __forceinline__ void staged_out(const TcArgs& args, const Geom& G, co
         asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
         __syncwarp();
         if (n0 < args.ep.n && tok0 < args.ep.m_tok && elect_one()) {
-            if (mode == OUT_ADD)
+            if (mode == OUT_ADD) {
                 tma_reduce(&args.map_o, smem_u32(sl), n0, tok0, 0);
-            else
+            } else if (mode == OUT_F32) {
                 tma_store(&args.map_o, smem_u32(sl), n0, tok0, 0);
+            } else {
+                tma_store(&args.map_o, smem_u32(sl), n0, tok0, 0);
+                if (nw > 16 && n0 + 16 < args.ep.n) tma_store(&args.map_o, smem_u32(sl) + CH * 32, n0 + 16, tok0, 0);
+            }
             asm volatile("cp.async.bulk.commit_group;" ::: "memory");
         }
         if (++slot == args.n_slots) slot = 0;
@@ -271,6 +277,7 @@ __global__ void __launch_bounds__(kThreads, 1) gemm_tc_kernel(const __grid_const
     G.bn = args.bn;
     G.n_bufs = args.n_bufs;
     G.pair = args.pair;
+    G.a_bytes = args.a_bytes;
     G.b_bytes = args.b_bytes;
     G.stage_bytes = args.stage_bytes;
     G.idesc = args.idesc;
@@ -339,10 +346,10 @@ __global__ void __launch_bounds__(kThreads, 1) gemm_tc_kernel(const __grid_const
             const bool evict_first = args.evict_first != 0;
             if (evict_first)
                 asm volatile("createpolicy.fractional.L2::evict_first.b64 %0, 1.0;" : "=l"(policy));
-            const uint32_t b_base = kABytes * G.n_a * G.kbs;
-            const uint32_t tx = kABytes * G.n_a + G.b_bytes;
+            const uint32_t b_base = G.a_bytes * G.n_a * G.kbs;
+            const uint32_t tx = G.a_bytes * G.n_a + G.b_bytes;
             // first weight row of a unit in both maps (a pair's second map starts 128 rows in)
-            const int row_step = kBM << G.pair;
+            const int row_step = args.bm << G.pair;
             // Weights do not depend on the previous kernel: the first ring of stages gets its
             // weight tiles before griddepcontrol.wait, the activation tiles after it.
             int pend_kx[kMaxStages], pend_nk[kMaxStages], pend_tok[kMaxStages], pend_grp[kMaxStages];
@@ -377,15 +384,15 @@ __global__ void __launch_bounds__(kThreads, 1) gemm_tc_kernel(const __grid_const
                     for (int j = 0; j < nk; ++j) {
                         const int kx = (kb + j) * kBK;
                         if (evict_first) {
-                            tma_load_3d_hint(st + j * kABytes, mA, kx, x.n_tile * row_step, x.group,
+                            tma_load_3d_hint(st + j * G.a_bytes, mA, kx, x.n_tile * row_step, x.group,
                                              full_bar(stage), policy);
                             if (G.n_a == 2)
-                                tma_load_3d_hint(st + (G.kbs + j) * kABytes, mA2, kx, x.n_tile * row_step,
+                                tma_load_3d_hint(st + (G.kbs + j) * G.a_bytes, mA2, kx, x.n_tile * row_step,
                                                  x.group, full_bar(stage), policy);
                         } else {
-                            tma_load_3d(st + j * kABytes, mA, kx, x.n_tile * row_step, x.group, full_bar(stage));
+                            tma_load_3d(st + j * G.a_bytes, mA, kx, x.n_tile * row_step, x.group, full_bar(stage));
                             if (G.n_a == 2)
-                                tma_load_3d(st + (G.kbs + j) * kABytes, mA2, kx, x.n_tile * row_step, x.group,
+                                tma_load_3d(st + (G.kbs + j) * G.a_bytes, mA2, kx, x.n_tile * row_step, x.group,
                                             full_bar(stage));
                         }
                     }
@@ -434,7 +441,7 @@ __global__ void __launch_bounds__(kThreads, 1) gemm_tc_kernel(const __grid_const
             int stage = 0, acc = 0;
             uint32_t phase = 0, acc_phase = 0;
             bool ok = true;
-            const uint32_t b_base = kABytes * G.n_a * G.kbs;
+            const uint32_t b_base = G.a_bytes * G.n_a * G.kbs;
             for (int u = blockIdx.x; u < G.n_units && ok; u += gridDim.x) {
                 const Unit x = decode_unit(G, u);
                 if (!bar_wait(tempty_bar(acc), acc_phase ^ 1u, abort_flag, err)) break;
@@ -449,8 +456,8 @@ __global__ void __launch_bounds__(kThreads, 1) gemm_tc_kernel(const __grid_const
                     tc_fence_after();
                     const uint32_t st = sbase + (uint32_t)stage * G.stage_bytes;
                     for (int j = 0; j < nk; ++j) {
-                        const uint64_t da = smem_desc(st + j * kABytes);
-                        const uint64_t da2 = smem_desc(st + (G.kbs + j) * kABytes);
+                        const uint64_t da = smem_desc(st + j * G.a_bytes);
+                        const uint64_t da2 = smem_desc(st + (G.kbs + j) * G.a_bytes);
                         const uint64_t db = smem_desc(st + b_base + j * G.b_bytes);
 #pragma unroll
                         for (int k = 0; k < kBK / 16; ++k) {
@@ -637,8 +644,8 @@ bool encode_tma_bf16(CUtensorMap* m, const void* base, int rank, const uint64_t*
                      const uint64_t* strides_bytes, const uint32_t* box) {
     return encode_tma(m, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, base, rank, dims, strides_bytes, box);
 }
-// boxes of 64-byte rows, packed
-static bool encode_tma_rows64(CUtensorMap* m, const void* base, const uint64_t* dims, const uint64_t* strides_bytes,
+// packed boxes (no swizzle)
+static bool encode_tma_packed(CUtensorMap* m, const void* base, const uint64_t* dims, const uint64_t* strides_bytes,
                               const uint32_t* box) {
     return encode_tma(m, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, base, 3, dims, strides_bytes, box, CU_TENSOR_MAP_SWIZZLE_NONE);
 }
@@ -681,7 +688,24 @@ cudaError_t launch_gemm_tc(dflare_ctx* c, const GemmDesc& g, cudaStream_t s, std
     }
     a.n_a = (g.a2 || a.pair) ? 2 : 1;
     a.tok_tiles = (g.m_tok + a.bn - 1) / a.bn;
-    a.n_tiles = (g.n + (kBM << a.pair) - 1) / (kBM << a.pair);
+    // SwiGLU tiles of fewer weight rows where that divides one wave better: its K splits would go through
+    // the workspace, and 128-row tiles leave a third of the SMs without any weights to stream (d 4096, ffn
+    // 12288: 96 tiles of 128, 128 of 96). The MMA still multiplies 128 rows; those past the tile's (whatever
+    // lies behind it in shared memory) end in accumulator lanes that nobody reads.
+    a.bm = kBM;
+    const bool swiglu_tma = g.ep.kind == EPI_SWIGLU && (reinterpret_cast<uintptr_t>(g.ep.out) & 15u) == 0 && g.ep.ldo % 8 == 0;
+    if (swiglu_tma && g.force_splits <= 0) {
+        long long best_cost = 0;
+        for (int bm = kBM; bm >= 64; bm -= 16) {
+            const long long t = (long long)g.groups * ((g.n + bm - 1) / bm) * a.tok_tiles;
+            const long long cost = (t + c->num_sms - 1) / c->num_sms * bm;
+            if (bm == kBM || cost < best_cost) {
+                best_cost = cost;
+                a.bm = bm;
+            }
+        }
+    }
+    a.n_tiles = (g.n + (a.bm << a.pair) - 1) / (a.bm << a.pair);
     a.k_blocks = (g.k + kBK - 1) / kBK;
     const int tiles = g.groups * a.n_tiles * a.tok_tiles;
     const int sms = c->num_sms;
@@ -713,7 +737,7 @@ cudaError_t launch_gemm_tc(dflare_ctx* c, const GemmDesc& g, cudaStream_t s, std
         a.out_mode = OUT_ADD;
     }
     if (g.ep.kind == EPI_RESID && !det && rows16(g.ep.resid, 4ll * g.ep.ld_resid)) a.out_mode = OUT_ADD;
-    if (g.ep.kind == EPI_SWIGLU && rows16(g.ep.out, 2ll * g.ep.ldo)) a.out_mode = OUT_SWIGLU;
+    if (swiglu_tma) a.out_mode = OUT_SWIGLU;
     if (g.ep.kind == EPI_F32 && !a.pair && rows16(g.ep.out, 4ll * g.ep.ldo)) a.out_mode = OUT_F32;
     const int ch = a.bn % 32 == 0 ? 32 : 16;   // tokens per staging slot
     a.n_slots = std::min(a.bn / ch, 64 / ch);
@@ -721,7 +745,9 @@ cudaError_t launch_gemm_tc(dflare_ctx* c, const GemmDesc& g, cudaStream_t s, std
                                                  : 4 * a.n_slots * ch * (a.out_mode == OUT_SWIGLU ? 64 : 128);
     a.epi_bytes = epi_bytes;
     const int misc_bytes = 16;
-    const int fixed = 1024 + epi_bytes + 8 * (2 * kMaxStages + 5) + misc_bytes;
+    // (128-row operand reads that start at a shorter tile end inside the allocation)
+    const int slack = (kBM - a.bm) * kBK * 2;
+    const int fixed = 1024 + epi_bytes + 8 * (2 * kMaxStages + 5) + misc_bytes + slack;
     const int budget = g.max_smem > 0 ? std::min(g.max_smem, kSmemLimit) : kSmemLimit;
     if (g.kbs > 0) {
         a.kbs = g.kbs;
@@ -731,8 +757,8 @@ cudaError_t launch_gemm_tc(dflare_ctx* c, const GemmDesc& g, cudaStream_t s, std
         // 64 tokens, d 4096: Q/K/V 11.7 / 11.5 / 12.4, down 20.0 / 19.1 / 21.0, gate/up - / 37.9 / 36.7; 32 tokens,
         // GPT-OSS gate/up - / 27.7 / 25.1; 16 tokens, d 2560: O 5.8 / 6.2 / 7.3. Gate/up at 16 tokens keeps its
         // three stages of two (Qwen3-4B block 422.8 -> 418.8).
-        const int kb_bytes = kBM * kBK * 2 * a.n_a + a.bn * kBK * 2;
-        a.kbs = a.n_a == 2 && a.bn == 16 ? 2 : 3 * 4 * kb_bytes <= budget - fixed ? 4 : 4 * 2 * kb_bytes <= budget - fixed ? 2 : 1;
+        const int kb_bytes = a.bm * kBK * 2 * a.n_a + a.bn * kBK * 2;
+        a.kbs = 3 * 4 * kb_bytes <= budget - fixed ? 4 : (a.bn == 16 ? 3 : 4) * 2 * kb_bytes <= budget - fixed ? 2 : 1;
     }
     if (g.force_splits > 0) best = std::min(g.force_splits, a.k_blocks);
     a.kb_per_split = (a.k_blocks + best - 1) / best;
@@ -746,14 +772,15 @@ cudaError_t launch_gemm_tc(dflare_ctx* c, const GemmDesc& g, cudaStream_t s, std
     }
     a.n_units = tiles * a.splits;
     a.b_bytes = (uint32_t)a.bn * kBK * 2;
-    a.stage_bytes = (uint32_t)a.kbs * (kABytes * a.n_a + a.b_bytes);
+    a.a_bytes = (uint32_t)a.bm * kBK * 2;
+    a.stage_bytes = (uint32_t)a.kbs * (a.a_bytes * a.n_a + a.b_bytes);
     a.evict_first = g.evict_first >= 0 ? 1 : 0;
     a.stages = std::min(kMaxStages, (budget - fixed) / (int)a.stage_bytes);
     if (a.stages < 2) {
         if (why) *why = "tcgen05 GEMM: tile does not fit in shared memory";
         return cudaErrorInvalidValue;
     }
-    const int smem = 1024 + a.stages * (int)a.stage_bytes + epi_bytes + 8 * (2 * a.stages + 5) + misc_bytes;
+    const int smem = 1024 + a.stages * (int)a.stage_bytes + epi_bytes + 8 * (2 * a.stages + 5) + misc_bytes + slack;
     a.n_bufs = (2 * a.n_a * a.bn <= 512) ? 2 : 1;
     int cols = 32;
     while (cols < a.n_bufs * a.n_a * a.bn) cols <<= 1;
@@ -781,8 +808,8 @@ cudaError_t launch_gemm_tc(dflare_ctx* c, const GemmDesc& g, cudaStream_t s, std
     // a pair's second tile: the same matrix from row 128 on (rows past its end read as zeros)
     const void* a2 = g.a2 ? g.a2 : a.pair ? static_cast<const void*>(static_cast<const bf16*>(g.a) + (size_t)kBM * g.k)
                                           : g.a;
-    if (!make_map(&a.map_a, g.a, g.k, g.n, g.groups, a_gr, kBM) ||
-        !make_map(&a.map_a2, a2, g.k, a.pair ? g.n - kBM : g.n, g.groups, a_gr, kBM) ||
+    if (!make_map(&a.map_a, g.a, g.k, g.n, g.groups, a_gr, a.bm) ||
+        !make_map(&a.map_a2, a2, g.k, a.pair ? g.n - kBM : g.n, g.groups, a_gr, a.bm) ||
         !make_map(&a.map_b, g.b, b_k, g.m_tok, b_groups, b_gr, a.bn)) {
         if (why) *why = "cuTensorMapEncodeTiled failed (alignment or driver entry point)";
         return cudaErrorInvalidValue;
@@ -791,9 +818,9 @@ cudaError_t launch_gemm_tc(dflare_ctx* c, const GemmDesc& g, cudaStream_t s, std
         const bool h16 = a.out_mode == OUT_SWIGLU;
         const uint64_t ld = h16 ? 2ull * g.ep.ldo : 4ull * (g.ep.kind == EPI_RESID ? g.ep.ld_resid : g.ep.ldo);
         const uint64_t dims[3] = {(uint64_t)g.n, (uint64_t)g.m_tok, 1}, st[2] = {ld, ld * (uint64_t)g.m_tok};
-        const uint32_t box[3] = {32, (uint32_t)ch, 1};
+        const uint32_t box[3] = {h16 ? 16u : 32u, (uint32_t)ch, 1};
         void* out = g.ep.kind == EPI_RESID ? static_cast<void*>(g.ep.resid) : g.ep.out;
-        if (!(h16 ? encode_tma_rows64(&a.map_o, out, dims, st, box) : encode_tma_f32(&a.map_o, out, 3, dims, st, box))) {
+        if (!(h16 ? encode_tma_packed(&a.map_o, out, dims, st, box) : encode_tma_f32(&a.map_o, out, 3, dims, st, box))) {
             if (why) *why = "cuTensorMapEncodeTiled failed (output)";
             return cudaErrorInvalidValue;
         }

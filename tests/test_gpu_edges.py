@@ -96,6 +96,19 @@ def test_two_sm_gemm_of_the_variants_matches_oracle(flag, kw, d):
     _step_matches_oracle(w, getattr(P, flag), **kw)
 
 
+# gate/up tiles of 80 (125 and 152 SMs' worth), 112 and 64 weight rows, token tiles of 16, 32 and 48 rows
+SWIGLU_CASES = [
+    synth.Workload("swiglu_9984", _shape(d=128, ffn=9984, block=9), (33,), 0.8, 61),
+    synth.Workload("swiglu_16960", _shape(d=128, ffn=16960, block=16), (20, 40), 0.8, 62),
+    synth.Workload("swiglu_9728", _shape(d=128, ffn=9728, block=11), (20, 40, 1, 7), 0.8, 63),
+]
+
+
+@pytest.mark.parametrize("w", SWIGLU_CASES, ids=lambda w: w.name)
+def test_gate_up_tiles_match_oracle(w):
+    _step_matches_oracle(w)
+
+
 # context fills of at least two positions per SM: one and two feature groups per thread (five and six draft
 # layers), two CTAs per SM, warps with and without their second group, target-layer counts that end inside
 # a stage of 6 (bf16) or 3 (fp32) rows, fewer target rows than a stage, positions past a sequence's end
