@@ -12,7 +12,7 @@
 // L1 limit. The earlier form (128 rows x 16 tokens per CTA, K in shared-memory chunks of 16 between
 // two barriers) waited a memory round trip per chunk (ncu: 32 us at K 256, 92 us at K 768). With this
 // kernel and the fp32 attention of attention.cu the first step of a 128-position sequence on the fp32
-// drafter (d 256, 4 layers, block 8) went from 968 to 153 us.
+// drafter (d 256, 4 layers, block 8) went from 968 to 158 us, and to 134 with two chunks of K per round.
 #include "epilogue.cuh"
 
 namespace dfl {
@@ -58,9 +58,15 @@ __global__ void __launch_bounds__(kSimtThreads) gemm_simt_kernel(
 #pragma unroll
     for (int f = 0; f < 4; ++f) wp[f] = Ag + (size_t)min(row0 + f, n - 1) * k + 4 * lane;   // rows past n: not stored
     const float4 zero = make_float4(0.f, 0.f, 0.f, 0.f);
-    float4 w[4];
+    // KC chunks of 128 k per round, whose loads are in flight together: the fp32 step above 158 us with one,
+    // 134 with two, 139 with three (254 registers: the next launch starts later; at 16 tokens a second
+    // chunk would spill)
+    constexpr int KC = TT == 8 ? 2 : 1;
+    float4 w[KC][4];
 #pragma unroll
-    for (int f = 0; f < 4; ++f) w[f] = 4 * lane < k ? ld4(wp[f]) : zero;
+    for (int j = 0; j < KC; ++j)
+#pragma unroll
+        for (int f = 0; f < 4; ++f) w[j][f] = 4 * lane + 128 * j < k ? ld4(wp[f] + 128 * j) : zero;
     pdl_wait();
     pdl_trigger();   // after the wait: see gemm_tc_kernel
     const T* Bg = Bm + (size_t)(b_shared || b_kgroup > 0 ? 0 : group) * b_group_rows * k;
@@ -68,33 +74,39 @@ __global__ void __launch_bounds__(kSimtThreads) gemm_simt_kernel(
     float acc[4 * TT];
 #pragma unroll
     for (int i = 0; i < 4 * TT; ++i) acc[i] = 0.f;
-    for (int c0 = 0; c0 < k; c0 += 128) {
-        const int col = c0 + 4 * lane;
-        const bool in = col < k;
-        const T* bp = Bg + col;
-        if (b_kgroup > 0) {   // contraction over stacked activation groups (Eq. 1)
-            const int z = col / b_kgroup;
-            bp = Bm + (size_t)z * b_group_rows * b_kgroup + (col - z * b_kgroup);
-        }
-        float4 x[TT];
+    for (int c0 = 0; c0 < k; c0 += 128 * KC) {
+        float4 x[KC][TT];
 #pragma unroll
-        for (int t = 0; t < TT; ++t) x[t] = in ? ld4(bp + (size_t)min(tok0 + t, m_tok - 1) * b_ld) : zero;
-        float4 wn[4];
-        const bool more = col + 128 < k;
-#pragma unroll
-        for (int f = 0; f < 4; ++f) wn[f] = more ? ld4(wp[f] + c0 + 128) : zero;
-#pragma unroll
-        for (int f = 0; f < 4; ++f)
-#pragma unroll
-            for (int t = 0; t < TT; ++t) {
-                float a = acc[f * TT + t];
-                a = fmaf(w[f].x, x[t].x, a);
-                a = fmaf(w[f].y, x[t].y, a);
-                a = fmaf(w[f].z, x[t].z, a);
-                acc[f * TT + t] = fmaf(w[f].w, x[t].w, a);
+        for (int j = 0; j < KC; ++j) {
+            const int col = c0 + 128 * j + 4 * lane;
+            const bool in = col < k;
+            const T* bp = Bg + col;
+            if (b_kgroup > 0) {   // contraction over stacked activation groups (Eq. 1)
+                const int z = col / b_kgroup;
+                bp = Bm + (size_t)z * b_group_rows * b_kgroup + (col - z * b_kgroup);
             }
 #pragma unroll
-        for (int f = 0; f < 4; ++f) w[f] = wn[f];
+            for (int t = 0; t < TT; ++t) x[j][t] = in ? ld4(bp + (size_t)min(tok0 + t, m_tok - 1) * b_ld) : zero;
+        }
+#pragma unroll
+        for (int j = 0; j < KC; ++j) {
+            float4 wn[4];
+            const int next = c0 + 128 * (KC + j);
+#pragma unroll
+            for (int f = 0; f < 4; ++f) wn[f] = next + 4 * lane < k ? ld4(wp[f] + next) : zero;
+#pragma unroll
+            for (int f = 0; f < 4; ++f)
+#pragma unroll
+                for (int t = 0; t < TT; ++t) {
+                    float a = acc[f * TT + t];
+                    a = fmaf(w[j][f].x, x[j][t].x, a);
+                    a = fmaf(w[j][f].y, x[j][t].y, a);
+                    a = fmaf(w[j][f].z, x[j][t].z, a);
+                    acc[f * TT + t] = fmaf(w[j][f].w, x[j][t].w, a);
+                }
+#pragma unroll
+            for (int f = 0; f < 4; ++f) w[j][f] = wn[f];
+        }
     }
     // add the 32 lanes' sums: at each step a lane keeps one half of its values (the upper half when
     // its lane bit is set) and gives the other away; afterwards it holds values 4 TT / 32 * lane ..
