@@ -242,11 +242,16 @@ __global__ void __launch_bounds__(256) spec_stats_kernel(const float* __restrict
             m = gm;
         }
         if (m > -INFINITY) {
+            float a[kU] = {};   // one chain of additions per group; a NaN adds nothing
 #pragma unroll
-            for (int g = 0; g < kU; ++g)
+            for (int e = 0; e < 4; ++e)
 #pragma unroll
-                for (int e = 0; e < 4; ++e)
-                    if (x[g][e] > -INFINITY) s += expf(x[g][e] - m);
+                for (int g = 0; g < kU; ++g) {
+                    const float t = expf(x[g][e] - m);
+                    a[g] += x[g][e] > -INFINITY ? t : 0.f;
+                }
+#pragma unroll
+            for (int g = 0; g < kU; ++g) s += a[g];
         }
     }
     __shared__ float sm[8], ss[8];

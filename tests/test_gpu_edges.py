@@ -73,6 +73,7 @@ def test_simt_gemm_on_bf16_matches_oracle():
 PAIR_CASES = [
     synth.Workload("pair_129", _shape(block=3, vocab=1003, ffn=192, d=320), tuple(3 + b % 5 for b in range(43)), 0.8, 41),
     synth.Workload("pair_192", _shape(block=32, vocab=1000, ffn=1088, d=320, n_q_heads=8), (40, 3, 33, 1, 17, 64), 0.8, 42),
+    synth.Workload("pair_160_odd_vocab", _shape(block=32, vocab=1003, ffn=320), (40, 3, 33, 1, 17), 0.8, 46),
     synth.Workload("pair_fill_257", _shape(head_dim=128, ffn=192), (257,), 0.8, 43),
     synth.Workload("pair_288", _shape(block=32, vocab=2004, head_dim=128, ffn=704, d=576), (300, 1, 2, 5, 257, 9, 3, 30, 64), 0.8, 44),
 ]
