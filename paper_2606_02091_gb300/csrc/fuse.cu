@@ -550,9 +550,9 @@ cudaError_t fuse_layers_t(dflare_ctx* c, const void* hidden, int n_max, void* fu
     const T* gain = static_cast<const T*>(c->w.fuse_norm);
     T* F = static_cast<T*>(c->fused);
     T* Fo = static_cast<T*>(fused_out);
-    // context fill: warp-specialised CTAs of d / 8 consumer threads and a producer warp, two per SM
-    // when their registers allow (rings of about 100 KB), else one (about 200 KB); at most kMaxNS
-    // stages of kRB rows
+    // context fill: CTAs of d / 8 threads (up to five draft layers) or d / 16 (six to eight, at least enough
+    // warps for a balanced SM), two per SM when their registers allow (rings of about 100 KB), else one
+    // (about 200 KB); at most kMaxNS stages
     const size_t stage_bytes = (size_t)kRowsPerStage<T> * g.d * sizeof(T);
     const int Dn = g.n_draft_layers, nf = Dn <= 5 ? 1 : 2;
     const int threads = std::min(512 / nf, (g.d / 8 + 31) / 32 * 32);   // (d <= 4096)

@@ -676,9 +676,9 @@ cudaError_t launch_gemm_tc(dflare_ctx* c, const GemmDesc& g, cudaStream_t s, std
     // the SwiGLU gate and up tiles do), a third fewer shared-memory bytes per FLOP. At 256 token
     // rows the pair fills all 512 TMEM columns, so a unit's epilogue no longer overlaps the next
     // unit's MMAs: pairs pay only for the cheap fp32-logit epilogue (the LM head), and only when
-    // their wave count times ~1.8 single-tile units beats the single tiles' wave count.
-    // Measured: batch-16 step 1.965 -> 1.947 ms (the LM head); the context fill's K/V projection
-    // with its rotary epilogue lost (Qwen3-4B shape 822 -> 640 TFLOP/s).
+    // their wave count times ~1.8 single-tile units beats the single tiles' wave count (batch-16
+    // step 1.965 -> 1.947 ms). The two-SM GEMM has taken these launches over except for vocabularies
+    // whose rows do not start on 16 bytes.
     {
         const long long u1 = (long long)g.groups * ((g.n + kBM - 1) / kBM) * ((g.m_tok + a.bn - 1) / a.bn);
         const long long u2 = (long long)g.groups * ((g.n + 2 * kBM - 1) / (2 * kBM)) * ((g.m_tok + a.bn - 1) / a.bn);
@@ -691,7 +691,9 @@ cudaError_t launch_gemm_tc(dflare_ctx* c, const GemmDesc& g, cudaStream_t s, std
     // SwiGLU tiles of fewer weight rows where that divides one wave better: its K splits would go through
     // the workspace, and 128-row tiles leave a third of the SMs without any weights to stream (d 4096, ffn
     // 12288: 96 tiles of 128, 128 of 96). The MMA still multiplies 128 rows; those past the tile's (whatever
-    // lies behind it in shared memory) end in accumulator lanes that nobody reads.
+    // lies behind it in shared memory) end in accumulator lanes that nobody reads. One launch, 128-row tiles
+    // -> these: 64 tokens, d 4096 (128 tiles of 96) 34.4 -> 33.3 us; 16 tokens, d 2560 (152 of 64, no K splits)
+    // 19.6 -> 18.0; 32 tokens, GPT-OSS (144 of 80) 24.3 -> 22.1.
     a.bm = kBM;
     const bool swiglu_tma = g.ep.kind == EPI_SWIGLU && (reinterpret_cast<uintptr_t>(g.ep.out) & 15u) == 0 && g.ep.ldo % 8 == 0;
     if (swiglu_tma && g.force_splits <= 0) {
