@@ -546,11 +546,12 @@ PairPlan plan_pair(const GemmDesc& g, int pairs, bool may_split) {
 
 bool gemm_pair_fits(const dflare_ctx* c, const GemmDesc& g) {
     const EpiParams& ep = g.ep;
-    // Against the single-SM GEMM at d 4096, ffn 12288 (us, single -> pair): 256 rows Q/K/V 19.5 -> 16.6,
-    // O 16.2 -> 14.2, gate/up 55.3 -> 38.2, down 31.3 -> 25.9, LM head (40000 entries) 102 -> 68; 192 rows
-    // 17.1 -> 16.5, -, 48.6 -> 37.9, 28.2 -> 25.8; 144 rows 13.7 -> 16.5, 11.6 -> 14.1, 43.3 -> 37.7, 21.8 -> 25.7,
-    // 72 -> 67 (135 rows): the projections that split K over all SMs cross over near 176 rows.
-    const int from = ep.kind == EPI_RESID || ep.kind == EPI_RED32 ? 176 : 128;
+    // Against the single-SM GEMM at d 4096, ffn 12288 (us, single -> pair): 256 rows Q/K/V 16.8 -> 16.6,
+    // O 14.2 -> 14.2, down 27.5 -> 25.9, gate/up 47.8 -> 38.0, LM head (40000 entries) 88.6 -> 68.3; 224 rows
+    // 16.1 -> 16.6, 13.5 -> 14.1, 26.2 -> 25.8, 44.8 -> 37.8, 84.7 -> 67.7; 144 rows 14.5 -> 16.5, 12.4 -> 14.1,
+    // 23.6 -> 25.6, 37.3 -> 37.6, 75.5 -> 67.0. The projections that split K over all SMs cross over near 224
+    // rows, the others at about 128 (gate/up of the Qwen3-4B shape, 144 rows: 23.0 -> 21.8).
+    const int from = ep.kind == EPI_RESID || ep.kind == EPI_RED32 ? 224 : 128;
     if (g.m_tok <= from || g.n % 4 != 0 || g.k % kPairBK != 0) return false;
     if ((g.m_tok + kPairTok - 1) / kPairTok > kPairMaxTokList) return false;
     switch (ep.kind) {
