@@ -548,10 +548,12 @@ bool gemm_pair_fits(const dflare_ctx* c, const GemmDesc& g) {
     const EpiParams& ep = g.ep;
     // Against the single-SM GEMM at d 4096, ffn 12288 (us, single -> pair): 256 rows Q/K/V 16.8 -> 16.6,
     // O 14.2 -> 14.2, down 27.5 -> 25.9, gate/up 47.8 -> 38.0, LM head (40000 entries) 88.6 -> 68.3; 224 rows
-    // 16.1 -> 16.6, 13.5 -> 14.1, 26.2 -> 25.8, 44.8 -> 37.8, 84.7 -> 67.7; 144 rows 14.5 -> 16.5, 12.4 -> 14.1,
-    // 23.6 -> 25.6, 37.3 -> 37.6, 75.5 -> 67.0. The projections that split K over all SMs cross over near 224
-    // rows, the others at about 128 (gate/up of the Qwen3-4B shape, 144 rows: 23.0 -> 21.8).
-    const int from = ep.kind == EPI_RESID || ep.kind == EPI_RED32 ? 224 : 128;
+    // 16.1 -> 16.6, 13.5 -> 14.1, 26.2 -> 25.8, 44.8 -> 37.8, 84.7 -> 67.7; 144 rows 13.9 -> 16.5, 11.7 -> 14.1,
+    // 22.2 -> 25.6, 37.3 -> 37.6, 64.6 -> 67.1. The projections that split K over all SMs cross over near 224
+    // rows, an LM head of several waves at 160 (65.8 -> 67.1, at 192 rows 77.8 -> 67.4), the others at about 128
+    // (gate/up of the Qwen3-4B shape, 144 rows: 23.0 -> 21.8; 4096 logits 21.6 -> 16.7).
+    const int from = ep.kind == EPI_RESID || ep.kind == EPI_RED32 ? 224
+                     : ep.kind == EPI_F32 && g.n >= 128 * c->num_sms ? 160 : 128;
     if (g.m_tok <= from || g.n % 4 != 0 || g.k % kPairBK != 0) return false;
     if ((g.m_tok + kPairTok - 1) / kPairTok > kPairMaxTokList) return false;
     switch (ep.kind) {

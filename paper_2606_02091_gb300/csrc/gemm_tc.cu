@@ -688,19 +688,22 @@ cudaError_t launch_gemm_tc(dflare_ctx* c, const GemmDesc& g, cudaStream_t s, std
     }
     a.n_a = (g.a2 || a.pair) ? 2 : 1;
     a.tok_tiles = (g.m_tok + a.bn - 1) / a.bn;
-    // SwiGLU tiles of fewer weight rows where that divides one wave better: its K splits would go through
+    // SwiGLU and logit tiles of fewer weight rows where that divides the waves better: its K splits would go through
     // the workspace, and 128-row tiles leave a third of the SMs without any weights to stream (d 4096, ffn
     // 12288: 96 tiles of 128, 128 of 96). The MMA still multiplies 128 rows; those past the tile's (whatever
     // lies behind it in shared memory) end in accumulator lanes that nobody reads. One launch, 128-row tiles
     // -> these: 64 tokens, d 4096 (128 tiles of 96) 34.4 -> 33.3 us; 16 tokens, d 2560 (152 of 64, no K splits)
-    // 19.6 -> 18.0; 32 tokens, GPT-OSS (144 of 80) 24.3 -> 22.1.
+    // 19.6 -> 18.0; 32 tokens, GPT-OSS (144 of 80) 24.3 -> 22.1. Likewise for logits, in steps of 32 rows: 40000
+    // entries (417 tiles of 96 in 3 waves instead of 313 of 128) at 48 tokens 62.6 -> 53.4.
     a.bm = kBM;
     const bool swiglu_tma = g.ep.kind == EPI_SWIGLU && (reinterpret_cast<uintptr_t>(g.ep.out) & 15u) == 0 && g.ep.ldo % 8 == 0;
-    if (swiglu_tma && g.force_splits <= 0) {
+    const bool f32_tma = g.ep.kind == EPI_F32 && !a.pair && (reinterpret_cast<uintptr_t>(g.ep.out) & 15u) == 0 && g.ep.ldo % 4 == 0;
+    if ((swiglu_tma || f32_tma) && g.force_splits <= 0) {
+        // (every tile counts four rows more for its hand-overs)
         long long best_cost = 0;
-        for (int bm = kBM; bm >= 64; bm -= 16) {
+        for (int bm = kBM; bm >= 64; bm -= swiglu_tma ? 16 : 32) {
             const long long t = (long long)g.groups * ((g.n + bm - 1) / bm) * a.tok_tiles;
-            const long long cost = (t + c->num_sms - 1) / c->num_sms * bm;
+            const long long cost = (t + c->num_sms - 1) / c->num_sms * (bm + 4);
             if (bm == kBM || cost < best_cost) {
                 best_cost = cost;
                 a.bm = bm;
@@ -740,9 +743,10 @@ cudaError_t launch_gemm_tc(dflare_ctx* c, const GemmDesc& g, cudaStream_t s, std
     }
     if (g.ep.kind == EPI_RESID && !det && rows16(g.ep.resid, 4ll * g.ep.ld_resid)) a.out_mode = OUT_ADD;
     if (swiglu_tma) a.out_mode = OUT_SWIGLU;
-    if (g.ep.kind == EPI_F32 && !a.pair && rows16(g.ep.out, 4ll * g.ep.ldo)) a.out_mode = OUT_F32;
+    if (f32_tma) a.out_mode = OUT_F32;
     const int ch = a.bn % 32 == 0 ? 32 : 16;   // tokens per staging slot
-    a.n_slots = std::min(a.bn / ch, 64 / ch);
+    // (one slot or two less at 144 tokens make room for a third stage of two k-blocks)
+    a.n_slots = std::min(a.bn / ch, (a.n_a == 1 && a.bn == 144 ? 32 : 64) / ch);
     const int epi_bytes = a.out_mode == OUT_REGS ? a.n_a * kChunk * 128 * 4
                                                  : 4 * a.n_slots * ch * (a.out_mode == OUT_SWIGLU ? 64 : 128);
     a.epi_bytes = epi_bytes;
@@ -755,12 +759,13 @@ cudaError_t launch_gemm_tc(dflare_ctx* c, const GemmDesc& g, cudaStream_t s, std
         a.kbs = g.kbs;
     } else {
         // a hand-off costs about 300 clocks whatever its bytes, and a ring of two stages runs dry: four
-        // 64-wide k-blocks where three stages fit, two where four fit, else one. Measured (us at 4 / 2 / 1):
-        // 64 tokens, d 4096: Q/K/V 11.7 / 11.5 / 12.4, down 20.0 / 19.1 / 21.0, gate/up - / 37.9 / 36.7; 32 tokens,
-        // GPT-OSS gate/up - / 27.7 / 25.1; 16 tokens, d 2560: O 5.8 / 6.2 / 7.3. Gate/up at 16 tokens keeps its
-        // three stages of two (Qwen3-4B block 422.8 -> 418.8).
+        // 64-wide k-blocks where three stages fit, two where three (of one weight tile) or four (of gate and
+        // up) fit, else one. Measured (us at 4 / 2 / 1): 64 tokens, d 4096: Q/K/V 11.7 / 11.5 / 12.4, down
+        // 20.0 / 19.1 / 21.0, gate/up - / 37.9 / 36.7; 96 tokens Q/K/V - / 11.9 / 12.8, down - / 20.1 / 22.0, LM head of
+        // 40000 entries - / 59.4 / 72.4; 32 tokens, GPT-OSS gate/up - / 27.7 / 25.1; 16 tokens, d 2560: O 5.8 / 6.2 /
+        // 7.3. Gate/up at 16 tokens keeps its three stages of two (Qwen3-4B block 422.8 -> 418.8).
         const int kb_bytes = a.bm * kBK * 2 * a.n_a + a.bn * kBK * 2;
-        a.kbs = 3 * 4 * kb_bytes <= budget - fixed ? 4 : (a.bn == 16 ? 3 : 4) * 2 * kb_bytes <= budget - fixed ? 2 : 1;
+        a.kbs = 3 * 4 * kb_bytes <= budget - fixed ? 4 : (a.n_a == 1 || a.bn == 16 ? 3 : 4) * 2 * kb_bytes <= budget - fixed ? 2 : 1;
     }
     if (g.force_splits > 0) best = std::min(g.force_splits, a.k_blocks);
     a.kb_per_split = (a.k_blocks + best - 1) / best;
