@@ -276,19 +276,16 @@ __global__ void __launch_bounds__(kPairThreads, 1) gemm_pair_kernel(const __grid
                 }
             }
             if (!waited) flush();
-            // no copy is still landing when the pair's CTAs leave: the even CTA waits for every
-            // stage (both CTAs' bytes); the odd one leaves with it at the cluster barrier
-            if (rank == 0) {
-                for (int s = 0; s < S; ++s)
-                    if (issued & (1u << s)) {
-                        volatile int never = 0;
-                        bar_wait(full_bar(s), (issued_phase >> s) & 1u, ok ? &never : abort_flag, err);
-                    }
-            } else if (!ok) {   // after a timeout: its own last copies have landed long before
-                const uint64_t t0 = globaltimer_ns();
-                while (globaltimer_ns() - t0 < 1000000ull) {
-                }
-            }
+            // No copy is still landing and no commit still arriving in this CTA's shared memory when it leaves: a
+            // stage's empty barrier completes after the MMAs that read both CTAs' copies of it (the odd CTA's
+            // copies complete on the even one's barrier), and the last commit arrives in both CTAs, of which the
+            // even one's issuing thread sees its own. The cluster barrier below orders what the threads of the
+            // pair did, not these arrivals. After a timeout some stages have no MMAs any more; one limit for all
+            // of them ends the wait.
+            volatile int never = 0;
+            for (int s = 0; s < S; ++s)
+                if (issued & (1u << s)) bar_wait_slow(empty_bar(s), (issued_phase >> s) & 1u, &never, err);
+            if (rank == 1) bar_wait_slow(drain_bar, 0, &never, err);
         }
     } else if (warp == 9) {
         if (rank == 0 && elect_one()) {
@@ -501,7 +498,7 @@ __global__ void __launch_bounds__(kPairThreads, 1) gemm_pair_kernel(const __grid
     __syncwarp();
     __syncthreads();
     if (tst && threadIdx.x == 0) atomicMax(tst + 2 * args.t_slots, (unsigned long long)globaltimer_ns());
-    // neither CTA leaves while the other's MMAs, commits or copies may touch its shared memory
+    // neither CTA leaves, or frees its tensor memory, while the other's threads or MMAs may touch it
     cluster_barrier();
     if (warp == 9) {
         tc_fence_after();

@@ -86,6 +86,27 @@ def test_two_sm_gemm_matches_oracle(w, flag):
     _step_matches_oracle(w, getattr(P, flag) if flag else 0)
 
 
+def test_two_sm_gemm_of_one_ring_repeats_exactly():
+    """Contractions of one to three k-blocks: every copy and commit of a launch belongs to its last ring, so
+    a CTA that left before they had arrived would let them into the next launch's shared memory. Blocks drafted
+    back to back with fixed sums hold the same bits, and the first agrees with the oracle."""
+    import torch
+    from paper_2606_02091_gb300 import FLAG_DETERMINISTIC
+    w = synth.Workload("pair_one_ring", _shape(d=64, ffn=192, vocab=1000, block=32), (300, 1, 2, 5, 257, 9, 3, 30, 64), 0.8, 47)
+    _step_matches_oracle(w, FLAG_DETERMINISTIC)
+    g = GpuSide(w, flags=FLAG_DETERMINISTIC)
+    g.fuse(w.ctx_lens, want_fused=False)
+    s, n = w.shape, 16
+    last = torch.tensor(synth.initial_tokens(w), device="cuda")
+    toks = torch.zeros((n, w.batch, s.block - 1), dtype=torch.int32, device="cuda")
+    logits = torch.zeros((n, w.batch, s.block - 1, s.vocab), dtype=torch.float32, device="cuda")
+    for i in range(n):
+        g.lib.draft_block(last, toks[i], logits[i])
+    torch.cuda.synchronize()
+    assert logits[0].any() and torch.equal(logits, logits[:1].expand_as(logits)) and torch.equal(toks, toks[:1].expand_as(toks))
+    assert g.lib.device_error() == 0
+
+
 @pytest.mark.parametrize("flag,kw", [("FLAG_FUSION_FC", dict(fusion_fc=True)), ("FLAG_DFLASH_FC", dict(dflash_fc=True)),
                                      ("FLAG_SHARED_KV", dict(shared_kv=True))], ids=lambda x: x if isinstance(x, str) else "")
 @pytest.mark.parametrize("d", [256, 320])
