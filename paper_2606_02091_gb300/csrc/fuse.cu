@@ -236,6 +236,14 @@ __device__ __forceinline__ bool fill_wait(uint32_t bar, uint32_t parity, volatil
     }
 }
 
+// Waits, within one limit for all of them, for the copies of a ring of ns slots whose next stage to read is the one
+// in slot st (its full barrier's phase: `phase`). A slot that was not refilled uses the limit up.
+__device__ __noinline__ void fill_drain(uint32_t full_bar0, int ns, int st, uint32_t phase, uint32_t* err) {
+    atomicOr(err, DFLARE_DEVERR_TIMEOUT);
+    volatile int never = 0;
+    for (int i = 0; i < ns; ++i) fill_wait(full_bar0 + 8u * i, i >= st ? phase : phase ^ 1u, &never);
+}
+
 // Two fp32 lanes in one 64-bit register: the fill's sums use the paired FMA (fma.rn.f32x2, each
 // lane rounded as a scalar fmaf), which halves the instructions of the 8 x D FMAs per row.
 typedef unsigned long long f32x2;
@@ -360,6 +368,7 @@ __device__ __forceinline__ void fuse_rows_body(
         int rst = -kLag;                       // slot to refill (negative: none yet)
         uint32_t phase = 0, rphase = 0;
         bool ok = true;
+        int bad = 0;
         f32x2 acc2[DMAX][4 * NF];
         // one target row, in G of the NF groups: a warp whose last group lies past d leaves it out
         const bool all_groups = NF == 1 || (warp * 32 + (NF - 1) * n_ct) * 8 < d;
@@ -471,7 +480,6 @@ __device__ __forceinline__ void fuse_rows_body(
             if ((lane & 3) == 0) red[par][warp][lane >> 2] = v[0];
             // one barrier a position: it also tells every consumer whether one of them timed out, so
             // that they leave together
-            int bad;
             asm volatile(
                 "{\n\t.reg .pred p, q;\n\t"
                 "setp.ne.s32 p, %1, 0;\n\t"
@@ -480,13 +488,7 @@ __device__ __forceinline__ void fuse_rows_body(
                 : "=r"(bad)
                 : "r"(ok ? 0 : 1), "r"(n_ct)
                 : "memory");
-            if (bad) {   // its copies in flight land long before the millisecond is over
-                if (tid == 0) atomicOr(err, DFLARE_DEVERR_TIMEOUT);
-                const uint64_t t0 = globaltimer_ns();
-                while (globaltimer_ns() - t0 < 1000000ull) {
-                }
-                break;
-            }
+            if (bad) break;
             // every warp adds the warps' sums itself: lane = value lane % 8, warps lane / 8, + 4, ...
             float tot = 0.f;
             for (int w = lane >> 3; w < n_cw; w += 4) tot += red[par][w][lane & 7];
@@ -519,6 +521,9 @@ __device__ __forceinline__ void fuse_rows_body(
                 if (i + kGP < DMAX) fetch_gain(i + kGP);
             }
         }
+        // after a timeout: the copies in flight, none beyond the stage that this thread reads next from their
+        // slot, land before the CTA leaves, within one more limit for all slots
+        if (bad && tid == 0) fill_drain(fb0, ns, st, phase, err);
     }
     __syncthreads();
 }
