@@ -54,3 +54,13 @@ def test_argmax_reads_the_mask_rows_logits_once():
     w = synth.preset("qwen3_4b")
     s = w.shape
     assert bench.algorithmic_bytes(w, "argmax", 6.0) == w.batch * (s.block - 1) * s.vocab * 4
+
+
+def test_event_timed_gemms_are_held_against_the_traced_step():
+    """The fp32 drafter's GEMMs, timed by event pairs: their sum holds the launches' latencies, so it may exceed
+    the step without events (153.9 us of pairs were seen beside a step of 132.9), but not the traced one."""
+    pairs = {"gemm_qkv": [0.0101] * 8, "gemm_o": [0.0095] * 8, "gemm_gate_up": [0.0092] * 8, "gemm_down": [0.00967] * 8}
+    us = bench.event_gemm_us(pairs, traced_ms=0.31, nb=2)
+    assert us == pytest.approx(1e3 * sum(sum(t) for t in pairs.values()) / 2) and us > 132.9
+    with pytest.raises(RuntimeError, match="traced step"):
+        bench.event_gemm_us(pairs, traced_ms=0.13, nb=2)
