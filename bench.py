@@ -27,6 +27,7 @@ import subprocess
 import sys
 import threading
 import time
+import traceback
 
 ROOT = os.path.dirname(os.path.abspath(__file__))
 sys.path.insert(0, ROOT)
@@ -1050,10 +1051,15 @@ def run_ours(args):
         for name in CONFIG_SET:
             if name == args.workload:
                 continue
-            sub = measure(synth.preset(name), args, args.steps, args.warmup, args.e2e_steps,
-                          args.breakdown_steps, 0.0 if args.no_cpu_baseline else args.sub_cpu_seconds,
-                          False, local=local)
-            line["configs"][name] = {k: sub[k] for k in SUB_KEYS if k in sub}
+            # a failed check of one of them is reported in its place; the headline stands by itself
+            try:
+                sub = measure(synth.preset(name), args, args.steps, args.warmup, args.e2e_steps,
+                              args.breakdown_steps, 0.0 if args.no_cpu_baseline else args.sub_cpu_seconds,
+                              False, local=local)
+                line["configs"][name] = {k: sub[k] for k in SUB_KEYS if k in sub}
+            except RuntimeError as e:
+                traceback.print_exc()
+                line["configs"][name] = {"error": f"{type(e).__name__}: {e}"}
     if rank == 0:
         print(json.dumps(line), flush=True)
     if dist:

@@ -64,3 +64,26 @@ def test_event_timed_gemms_are_held_against_the_traced_step():
     assert us == pytest.approx(1e3 * sum(sum(t) for t in pairs.values()) / 2) and us > 132.9
     with pytest.raises(RuntimeError, match="traced step"):
         bench.event_gemm_us(pairs, traced_ms=0.13, nb=2)
+
+
+def test_a_failed_configuration_leaves_the_headline(monkeypatch, capsys):
+    """One JSON line with the headline's value also when a further configuration's measurement fails."""
+    import json
+    import sys
+
+    import torch
+
+    def measure(w, *a, **kw):
+        if w.name == "tiny_f32":
+            raise RuntimeError("GEMM time exceeds the step")
+        return {"value": 1.5, "unit": bench.UNIT, "config": {"workload": w.name}}
+
+    monkeypatch.setattr(torch.cuda, "set_device", lambda i: None)
+    monkeypatch.setattr(bench, "measure", measure)
+    monkeypatch.setattr(sys, "argv", ["bench.py"])
+    assert bench.main() in (0, None)
+    out = capsys.readouterr().out.strip().splitlines()
+    line = json.loads(out[0])
+    assert len(out) == 1 and line["value"] == 1.5
+    assert "GEMM time" in line["configs"]["tiny_f32"]["error"]
+    assert all(line["configs"][n]["value"] == 1.5 for n in bench.CONFIG_SET if n not in ("tiny_f32", bench.HEADLINE))
