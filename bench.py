@@ -255,10 +255,15 @@ class Cudart:
         return ms.value
 
 
-def kernels_per_trace(shape):
-    """Kernel launches behind one traced call site (attention is one launch in bf16, split +
-    combine in fp32)."""
-    return {"attention": 1 if shape.dtype == "bf16" else 2}
+def kernels_per_trace(shape, batch, len_ub, num_sms):
+    """Kernel launches behind one traced call site. The fp32 attention has a second (combine) launch where it
+    splits the keys: beyond three tiles of 64 at the library's bound len_ub of the contexts, unless the 16-row
+    query tiles alone give every SM two CTAs."""
+    if shape.dtype == "bf16":
+        return {"attention": 1}
+    q_tiles = -(-shape.block * (shape.n_q_heads // shape.n_kv_heads) // 16)
+    split = -(-(len_ub + shape.block) // 64) > 3 and batch * shape.n_kv_heads * q_tiles < 2 * num_sms
+    return {"attention": 2 if split else 1}
 
 
 def algorithmic_bytes(w, name, mean_tau, mean_ctx=None):
@@ -689,32 +694,32 @@ def measure(w, args, steps, warmup, e2e_steps, nb, cpu_seconds, extras, dist=Non
     tgt = torch.zeros((w.batch, s.block), dtype=torch.int32, device="cuda")
     thr = synth.accept_threshold(w.match_p)
 
+    # the library's bound of the contexts: every fusion call adds its row stride
+    len_ub = min(max_ctx, len(fill_chunks) * chunk)
+
     def step_on(hid):
         def step():
+            nonlocal len_ub
             lib.fuse_context(hid, acc)
+            len_ub = min(max_ctx, len_ub + s.block)
             lib.draft_block(nxt, draft)
             synthetic_target(draft, u_d, r_d, last_d, step_ctr, thr, w.batch, s.block, tgt)
             lib.verify_accept(draft, tgt, acc, nxt)
         return step
 
-    # launch counting through the trace hook
-    counts = {}
+    # launch counting through the trace hook, while each of the timed graphs is captured
+    counts = [0]
+    num_sms = torch.cuda.get_device_properties(local).multi_processor_count
 
     @P._lib.TRACE_FN
     def count_cb(user, name, phase, stream):
         if phase == 0:
-            n = name.decode()
-            counts[n] = counts.get(n, 0) + 1
+            counts[-1] += kernels_per_trace(s, w.batch, len_ub, num_sms).get(name.decode(), 1)
 
     L_ = P.load()
-    L_.dflare_set_trace(lib.raw, count_cb, None)
     for i in range(3):
         step_on(hid_dev[i % N_ROT])()
     torch.cuda.synchronize()
-    kpt = kernels_per_trace(s)
-    launches_per_step = sum(kpt.get(k, 1) * v for k, v in counts.items()) / 3 + 1
-    L_.dflare_set_trace(lib.raw, P._lib.TRACE_FN(), None)
-
     cs = torch.cuda.Stream()
     cs.wait_stream(torch.cuda.current_stream())
     graphs = []
@@ -723,9 +728,13 @@ def measure(w, args, steps, warmup, e2e_steps, nb, cpu_seconds, extras, dist=Non
             g = torch.cuda.CUDAGraph()
             step_on(h)()
             torch.cuda.synchronize()
+            counts.append(1)   # the synthetic target, which the hook does not see
+            L_.dflare_set_trace(lib.raw, count_cb, None)
             with torch.cuda.graph(g, stream=cs):
                 step_on(h)()
+            L_.dflare_set_trace(lib.raw, P._lib.TRACE_FN(), None)
             graphs.append(g)
+    launches_per_step = sum(counts[1 + i % N_ROT] for i in range(K)) / K
     torch.cuda.synchronize()
     for i in range(Wm):
         graphs[i % N_ROT].replay()

@@ -87,3 +87,12 @@ def test_a_failed_configuration_leaves_the_headline(monkeypatch, capsys):
     assert len(out) == 1 and line["value"] == 1.5
     assert "GEMM time" in line["configs"]["tiny_f32"]["error"]
     assert all(line["configs"][n]["value"] == 1.5 for n in bench.CONFIG_SET if n not in ("tiny_f32", bench.HEADLINE))
+
+
+def test_launches_behind_the_fp32_attention():
+    """One launch up to three 64-key tiles (184 cached positions and a block of 8), a combine launch beyond, none
+    when 304 query tiles fill 152 SMs twice; bf16 always one."""
+    s = synth.preset("tiny_f32").shape
+    assert [bench.kernels_per_trace(s, 1, n, 152)["attention"] for n in (128, 184, 185, 4000)] == [1, 1, 2, 2]
+    assert bench.kernels_per_trace(s, 152, 4000, 152)["attention"] == 1
+    assert bench.kernels_per_trace(synth.preset("qwen3_4b").shape, 1, 4000, 152)["attention"] == 1
