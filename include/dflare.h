@@ -298,7 +298,9 @@ dflare_status dflare_device_error(dflare_ctx* ctx, uint32_t* bits_host, void* st
  * `stream` (name: "fuse_begin", "fuse_layers", "gemm_fusion_fc", "gemm_dflash_fc",
  * "gemm_kv_ctx", "embed", "rmsnorm", "gemm_qkv",
  * "attention", "gemm_o", "gemm_gate_up", "gemm_down", "gemm_lm_head", "argmax", "sample",
- * "argmax_target" (with the acceptance), "verify", "spec_stats", "spec_resample").
+ * "argmax_target", "verify", "spec_stats", "spec_accept", "spec_resample"). Two phases bracket no
+ * launch: "verify" in dflare_verify_logits, whose acceptance is the end of the "argmax_target"
+ * launch, and "spec_accept", which is the beginning of the "spec_resample" launch.
  * A caller can record CUDA events there, also while the stream is being captured into a graph.
  * fn = NULL turns tracing off. */
 typedef void (*dflare_trace_fn)(void* user, const char* name, int phase, void* stream);

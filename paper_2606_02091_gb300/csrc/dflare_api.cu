@@ -742,8 +742,11 @@ dflare_status dflare_verify_logits(dflare_ctx* c, const int32_t* draft, const fl
     if (reinterpret_cast<uintptr_t>(target_logits) % 16)
         return fail(c, DFLARE_EINVAL, "target_logits must be 16-byte aligned");
     cudaStream_t s = static_cast<cudaStream_t>(stream);
-    Trace t(c, "argmax_target", s);
-    CUDA_TRY(launch_argmax_verify(c, target_logits, draft, accept_len, next_token, s));
+    {
+        Trace t(c, "argmax_target", s);
+        CUDA_TRY(launch_argmax_verify(c, target_logits, draft, accept_len, next_token, s));
+    }
+    Trace t(c, "verify", s);   // a phase of its own for the caller, without a launch: see dflare_set_trace
     return DFLARE_OK;
 }
 
@@ -762,6 +765,9 @@ dflare_status dflare_verify_sampled(dflare_ctx* c, const int32_t* draft, const f
     {
         Trace t(c, "spec_stats", s);
         CUDA_TRY(launch_spec_stats(c, target_logits, inv_t, s));
+    }
+    {
+        Trace t(c, "spec_accept", s);   // likewise
     }
     Trace t(c, "spec_resample", s);
     CUDA_TRY(launch_spec_resample(c, draft, target_logits, inv_t, seed, step, accept_len, next_token, s));

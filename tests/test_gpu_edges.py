@@ -174,3 +174,30 @@ def test_copies_to_aligned_and_unaligned_buffers_agree(vocab, block, sampled):
         assert got[-1][2].any() and (block == 1 or got[-1][1].all())
     for a, b in zip(*got):
         np.testing.assert_array_equal(a, b)
+
+
+def test_verification_reports_every_phase():
+    """The trace hook sees the phases of the verification calls, also those whose work another launch does."""
+    import torch
+    import paper_2606_02091_gb300 as P
+    w = synth.Workload("phases", _shape(), (9, 4), 0.8, 37)
+    g, s, seen = GpuSide(w), w.shape, []
+    g.fuse(w.ctx_lens, want_fused=False)
+    g.draft(synth.initial_tokens(w))
+
+    @P._lib.TRACE_FN
+    def hook(user, name, phase, stream):
+        seen.append((name.decode(), phase))
+
+    drafts = torch.zeros((w.batch, s.block - 1), dtype=torch.int32, device="cuda")
+    target = torch.randn((w.batch, s.block, s.vocab), device="cuda")
+    acc, nxt = (torch.zeros(w.batch, dtype=torch.int32, device="cuda") for _ in range(2))
+    step = torch.zeros(1, dtype=torch.int64, device="cuda")
+    P.load().dflare_set_trace(g.lib.raw, hook, None)
+    g.lib.verify_logits(drafts, target, acc, nxt)
+    assert seen == [(n, p) for n in ("argmax_target", "verify") for p in (0, 1)]
+    seen.clear()
+    g.lib.verify_sampled(drafts, target, 1.0, 7, step, acc, nxt)
+    assert seen == [(n, p) for n in ("spec_stats", "spec_accept", "spec_resample") for p in (0, 1)]
+    P.load().dflare_set_trace(g.lib.raw, P._lib.TRACE_FN(), None)
+    torch.cuda.synchronize()
