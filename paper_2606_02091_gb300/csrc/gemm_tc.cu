@@ -428,11 +428,12 @@ __global__ void __launch_bounds__(kThreads, 1) gemm_tc_kernel(const __grid_const
                     load_b(sbase + pend_st[i] * G.stage_bytes, pend_kx[i], pend_nk[i], pend_tok[i],
                            pend_grp[i], full_bar(pend_st[i]));
             }
-            // no copy is still landing in shared memory when the CTA exits, after a timeout either (one
-            // more limit for all stages)
-            volatile int never = 0;
+            // no copy is still landing in shared memory when the CTA exits, after a timeout either
             for (int s = 0; s < S; ++s)
-                if (issued & (1u << s)) bar_wait(full_bar(s), (issued_phase >> s) & 1u, &never, err);
+                if (issued & (1u << s)) {
+                    volatile int never = 0;
+                    bar_wait(full_bar(s), (issued_phase >> s) & 1u, &never, err);
+                }
         }
     } else if (warp == 5) {
         if (elect_one()) {
