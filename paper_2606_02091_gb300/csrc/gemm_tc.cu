@@ -759,13 +759,14 @@ cudaError_t launch_gemm_tc(dflare_ctx* c, const GemmDesc& g, cudaStream_t s, std
         a.kbs = g.kbs;
     } else {
         // a hand-off costs about 300 clocks whatever its bytes, and a ring of two stages runs dry: four
-        // 64-wide k-blocks where three stages fit, two where three (of one weight tile) or four (of gate and
-        // up) fit, else one. Measured (us at 4 / 2 / 1): 64 tokens, d 4096: Q/K/V 11.7 / 11.5 / 12.4, down
-        // 20.0 / 19.1 / 21.0, gate/up - / 37.9 / 36.7; 96 tokens Q/K/V - / 11.9 / 12.8, down - / 20.1 / 22.0, LM head of
-        // 40000 entries - / 59.4 / 72.4; 32 tokens, GPT-OSS gate/up - / 27.7 / 25.1; 16 tokens, d 2560: O 5.8 / 6.2 /
-        // 7.3. Gate/up at 16 tokens keeps its three stages of two (Qwen3-4B block 422.8 -> 418.8).
+        // 64-wide k-blocks a stage where three stages fit, else two where three fit, else one. Measured (us
+        // after the dependency at 4 / 2 / 1): 64 tokens, d 4096: Q/K/V 11.7 / 11.5 / 12.4, down 20.0 / 19.1 / 21.0; 96
+        // tokens Q/K/V - / 11.9 / 12.8, down - / 20.1 / 22.0, LM head of 40000 entries - / 59.4 / 72.4; 16 tokens, d 2560:
+        // O 5.8 / 6.2 / 7.3. Gate/up at 2 / 1: 16 tokens, d 4096, ffn 16384 41.6 / 43.9, d 2560, ffn 19456 30.5 / 31.7; 32
+        // tokens 31.6 / 33.3; 64 tokens, d 4096, ffn 12288 34.4 / 35.1, d 2880, ffn 11520 23.6 / 24.3; 96 tokens, d 2560,
+        // ffn 9728 19.8 / 22.0.
         const int kb_bytes = a.bm * kBK * 2 * a.n_a + a.bn * kBK * 2;
-        a.kbs = 3 * 4 * kb_bytes <= budget - fixed ? 4 : (a.n_a == 1 || a.bn == 16 ? 3 : 4) * 2 * kb_bytes <= budget - fixed ? 2 : 1;
+        a.kbs = 3 * 4 * kb_bytes <= budget - fixed ? 4 : 3 * 2 * kb_bytes <= budget - fixed ? 2 : 1;
     }
     if (g.force_splits > 0) best = std::min(g.force_splits, a.k_blocks);
     a.kb_per_split = (a.k_blocks + best - 1) / best;

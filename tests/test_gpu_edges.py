@@ -118,11 +118,14 @@ def test_two_sm_gemm_of_the_variants_matches_oracle(flag, kw, d):
     _step_matches_oracle(w, getattr(P, flag), **kw)
 
 
-# gate/up tiles of 80 (125 and 152 SMs' worth), 112 and 64 weight rows, token tiles of 16, 32 and 48 rows
+# gate/up tiles of 80 (125 and 152 SMs' worth), 112, 64 and 96 weight rows, token tiles of 16, 32, 48 and 64 rows (one
+# and two of them), stages of four and of two k-blocks, the last one partly filled
 SWIGLU_CASES = [
     synth.Workload("swiglu_9984", _shape(d=128, ffn=9984, block=9), (33,), 0.8, 61),
     synth.Workload("swiglu_16960", _shape(d=128, ffn=16960, block=16), (20, 40), 0.8, 62),
     synth.Workload("swiglu_9728", _shape(d=128, ffn=9728, block=11), (20, 40, 1, 7), 0.8, 63),
+    synth.Workload("swiglu_12288", _shape(d=192, ffn=12288, block=16), (20, 40, 1, 7), 0.8, 64),
+    synth.Workload("swiglu_6144", _shape(d=448, ffn=6144, block=24), (20, 40, 1, 7, 3), 0.8, 65),
 ]
 
 
