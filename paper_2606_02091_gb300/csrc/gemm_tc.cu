@@ -745,16 +745,22 @@ cudaError_t launch_gemm_tc(dflare_ctx* c, const GemmDesc& g, cudaStream_t s, std
     if (swiglu_tma) a.out_mode = OUT_SWIGLU;
     if (f32_tma) a.out_mode = OUT_F32;
     const int ch = a.bn % 32 == 0 ? 32 : 16;   // tokens per staging slot
-    // (one slot or two less at 144 tokens make room for a third stage of two k-blocks)
-    a.n_slots = std::min(a.bn / ch, (a.n_a == 1 && a.bn == 144 ? 32 : 64) / ch);
-    const int epi_bytes = a.out_mode == OUT_REGS ? a.n_a * kChunk * 128 * 4
-                                                 : 4 * a.n_slots * ch * (a.out_mode == OUT_SWIGLU ? 64 : 128);
-    a.epi_bytes = epi_bytes;
+    const int kb_bytes = a.bm * kBK * 2 * a.n_a + a.bn * kBK * 2;   // one k-block of a stage
     const int misc_bytes = 16;
     // (128-row operand reads that start at a shorter tile end inside the allocation)
     const int slack = (kBM - a.bm) * kBK * 2;
-    const int fixed = 1024 + epi_bytes + 8 * (2 * kMaxStages + 5) + misc_bytes + slack;
     const int budget = g.max_smem > 0 ? std::min(g.max_smem, kSmemLimit) : kSmemLimit;
+    auto epi_of = [&](int slots) {
+        return a.out_mode == OUT_REGS ? a.n_a * kChunk * 128 * 4 : 4 * slots * ch * (a.out_mode == OUT_SWIGLU ? 64 : 128);
+    };
+    auto fixed_of = [&](int slots) { return 1024 + epi_of(slots) + 8 * (2 * kMaxStages + 5) + misc_bytes + slack; };
+    // staging for 64 tokens; for 32 where only that leaves room for a third stage of two k-blocks. One launch,
+    // 64 -> 32: 144 tokens, d 4096: O 12.7 -> 11.1 us, down 22.9 -> 21.8; 155 logit rows of 40000 entries 74.2 -> 68.3.
+    // (Where the ring stays the same, 32 cost up to 0.5 us: Q/K/V at 160 tokens 13.3 -> 13.7.)
+    a.n_slots = std::min(a.bn / ch, 64 / ch);
+    if (6 * kb_bytes > budget - fixed_of(a.n_slots) && 6 * kb_bytes <= budget - fixed_of(32 / ch)) a.n_slots = 32 / ch;
+    const int epi_bytes = epi_of(a.n_slots), fixed = fixed_of(a.n_slots);
+    a.epi_bytes = epi_bytes;
     if (g.kbs > 0) {
         a.kbs = g.kbs;
     } else {
@@ -765,7 +771,6 @@ cudaError_t launch_gemm_tc(dflare_ctx* c, const GemmDesc& g, cudaStream_t s, std
         // O 5.8 / 6.2 / 7.3. Gate/up at 2 / 1: 16 tokens, d 4096, ffn 16384 41.6 / 43.9, d 2560, ffn 19456 30.5 / 31.7; 32
         // tokens 31.6 / 33.3; 64 tokens, d 4096, ffn 12288 34.4 / 35.1, d 2880, ffn 11520 23.6 / 24.3; 96 tokens, d 2560,
         // ffn 9728 19.8 / 22.0.
-        const int kb_bytes = a.bm * kBK * 2 * a.n_a + a.bn * kBK * 2;
         a.kbs = 3 * 4 * kb_bytes <= budget - fixed ? 4 : 3 * 2 * kb_bytes <= budget - fixed ? 2 : 1;
     }
     if (g.force_splits > 0) best = std::min(g.force_splits, a.k_blocks);

@@ -134,6 +134,20 @@ def test_gate_up_tiles_match_oracle(w):
     _step_matches_oracle(w)
 
 
+# logit tiles of 96 and 64 weight rows, the last of 4, 36 and 64; 15, 60 and 155 token rows, the last with staging
+# for 32 tokens in place of 64
+LOGIT_CASES = [
+    synth.Workload("logits_14500", _shape(d=192, n_draft_layers=1, vocab=14500, block=16), (20,), 0.8, 71),
+    synth.Workload("logits_9700", _shape(d=192, n_draft_layers=1, vocab=9700, block=16), (20, 40, 1, 7), 0.8, 72),
+    synth.Workload("logits_40000", _shape(d=192, n_draft_layers=1, vocab=40000, block=32), (20, 40, 1, 7, 3), 0.8, 73),
+]
+
+
+@pytest.mark.parametrize("w", LOGIT_CASES, ids=lambda w: w.name)
+def test_logit_tiles_match_oracle(w):
+    _step_matches_oracle(w)
+
+
 # context fills of at least two positions per SM: one and two feature groups per thread (five and six draft
 # layers), two CTAs per SM, warps with and without their second group, target-layer counts that end inside
 # a stage of 6 (bf16) or 3 (fp32) rows, fewer target rows than a stage, positions past a sequence's end
