@@ -519,13 +519,11 @@ PairPlan plan_pair(const GemmDesc& g, int pairs, bool may_split) {
     PairPlan best{step, 1, kb};
     double best_t = 1e30;
     for (int bn = step; bn <= 256; bn += step) {
-        if (g.force_bn > 0 && bn != g.force_bn) continue;
         const long long tiles = (long long)g.groups * ((g.n + bn - 1) / bn) * tt;
         const double per_kb = std::max(4.0 * n_a * std::max(bn / 2, 64), (16384.0 + n_a * bn * 64.0) / 60.0);
         const bool overlap = 2 * n_a * bn <= 512;
         const double epi = 1500.0 + 12.0 * bn * n_a;
         for (int sp = 1; sp <= (may_split ? 8 : 1) && sp <= kb / 4 + 1; ++sp) {
-            if (g.force_splits > 0 && sp != g.force_splits) continue;
             const int kbp = (kb + sp - 1) / sp, spn = (kb + kbp - 1) / kbp;
             const long long waves = (tiles * spn + pairs - 1) / pairs;
             const double main = kbp * per_kb;
@@ -587,13 +585,17 @@ cudaError_t launch_gemm_pair(dflare_ctx* c, const GemmDesc& g, cudaStream_t s, s
     const int fixed = 1024 + kPairEpiWarps * (int)kBoxBytes + 8 * (2 * kPairMaxStages + 5) + 16 +
                       (a.compact ? 4 * a.tok_tiles : 0);
     const int budget = kPairSmemLimit - fixed;
-    a.kbs = g.kbs > 0 ? g.kbs : budget / (int)(2 * kb_bytes) >= 3 ? 2 : 1;
+    a.kbs = budget / (int)(2 * kb_bytes) >= 3 ? 2 : 1;
     if (g.b_kgroup > 0 && g.b_kgroup / kPairBK % a.kbs != 0) a.kbs = 1;   // a copy stays within one token group
     a.stage_bytes = kb_bytes * (uint32_t)a.kbs;
     a.stages = std::min(kPairMaxStages, budget / (int)a.stage_bytes);
+    if (a.stages < 2) {
+        if (why) *why = "two-SM GEMM: tile does not fit in shared memory";
+        return cudaErrorInvalidValue;
+    }
     a.n_bufs = 2 * a.n_a * a.bn <= 512 ? 2 : 1;
     // tokens that pass once leave their weights no second reader
-    a.evict_first = a.tok_tiles == 1 && g.evict_first >= 0;
+    a.evict_first = a.tok_tiles == 1;
     // kind::f16 instruction descriptor: fp32 accumulate, bf16 A and B, both K-major, N = bn, M = 256
     a.idesc = (1u << 4) | (1u << 7) | (1u << 10) | ((uint32_t)(a.bn >> 3) << 17) | ((256u >> 4) << 24);
     a.t_kg = g.b_kgroup / kPairBK;

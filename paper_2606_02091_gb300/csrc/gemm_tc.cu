@@ -68,7 +68,6 @@ struct TcArgs {
                                // (the second accumulator takes rows 128..255 of the pair)
     int kbs;                   // 64-wide k-blocks per pipeline stage
     uint32_t b_bytes;          // bytes of one activation sub-tile (bn x 64 bf16)
-    int evict_first;           // stream the weights with an L2 evict-first policy
     uint32_t idesc;
     uint32_t stage_bytes;
     float* ws;
@@ -343,9 +342,7 @@ __global__ void __launch_bounds__(kThreads, 1) gemm_tc_kernel(const __grid_const
             uint32_t phase = 0, issued = 0, issued_phase = 0;
             bool ok = true;
             uint64_t policy = 0;
-            const bool evict_first = args.evict_first != 0;
-            if (evict_first)
-                asm volatile("createpolicy.fractional.L2::evict_first.b64 %0, 1.0;" : "=l"(policy));
+            asm volatile("createpolicy.fractional.L2::evict_first.b64 %0, 1.0;" : "=l"(policy));
             const uint32_t b_base = G.a_bytes * G.n_a * G.kbs;
             const uint32_t tx = G.a_bytes * G.n_a + G.b_bytes;
             // first weight row of a unit in both maps (a pair's second map starts 128 rows in)
@@ -383,18 +380,10 @@ __global__ void __launch_bounds__(kThreads, 1) gemm_tc_kernel(const __grid_const
                     mbar_expect_tx(full_bar(stage), (uint32_t)nk * tx);
                     for (int j = 0; j < nk; ++j) {
                         const int kx = (kb + j) * kBK;
-                        if (evict_first) {
-                            tma_load_3d_hint(st + j * G.a_bytes, mA, kx, x.n_tile * row_step, x.group,
+                        tma_load_3d_hint(st + j * G.a_bytes, mA, kx, x.n_tile * row_step, x.group, full_bar(stage), policy);
+                        if (G.n_a == 2)
+                            tma_load_3d_hint(st + (G.kbs + j) * G.a_bytes, mA2, kx, x.n_tile * row_step, x.group,
                                              full_bar(stage), policy);
-                            if (G.n_a == 2)
-                                tma_load_3d_hint(st + (G.kbs + j) * G.a_bytes, mA2, kx, x.n_tile * row_step,
-                                                 x.group, full_bar(stage), policy);
-                        } else {
-                            tma_load_3d(st + j * G.a_bytes, mA, kx, x.n_tile * row_step, x.group, full_bar(stage));
-                            if (G.n_a == 2)
-                                tma_load_3d(st + (G.kbs + j) * G.a_bytes, mA2, kx, x.n_tile * row_step, x.group,
-                                            full_bar(stage));
-                        }
                     }
                     if (waited) {
                         load_b(st, kb * kBK, nk, x.tok_tile, x.group, full_bar(stage));
@@ -668,7 +657,7 @@ cudaError_t launch_gemm_tc(dflare_ctx* c, const GemmDesc& g, cudaStream_t s, std
     const bool ws_splits = g.ep.kind != EPI_RED32 && !(g.ep.kind == EPI_RESID && !(c->cfg.flags & DFLARE_FLAG_DETERMINISTIC));
     const long long w_tiles = (long long)g.groups * ((g.n + kBM - 1) / kBM);
     // (DFlash's FC keeps K splits: its contraction of T d is long enough to outweigh the partials)
-    while (ws_splits && g.force_splits <= 0 && g.b_kgroup == 0 && a.bn >= 128 &&
+    while (ws_splits && g.b_kgroup == 0 && a.bn >= 128 &&
            w_tiles * ((g.m_tok + a.bn / 2 - 1) / (a.bn / 2)) <= c->num_sms)
         a.bn = (a.bn / 2 + 15) / 16 * 16;
     // With token tiles of 128 or more rows the GEMM is bound by the tensor pipeline, not by HBM:
@@ -683,7 +672,7 @@ cudaError_t launch_gemm_tc(dflare_ctx* c, const GemmDesc& g, cudaStream_t s, std
         const long long u1 = (long long)g.groups * ((g.n + kBM - 1) / kBM) * ((g.m_tok + a.bn - 1) / a.bn);
         const long long u2 = (long long)g.groups * ((g.n + 2 * kBM - 1) / (2 * kBM)) * ((g.m_tok + a.bn - 1) / a.bn);
         const long long w1 = (u1 + c->num_sms - 1) / c->num_sms, w2 = (u2 + c->num_sms - 1) / c->num_sms;
-        a.pair = (!g.a2 && a.bn >= 128 && g.n > kBM && g.force_splits <= 0 &&
+        a.pair = (!g.a2 && a.bn >= 128 && g.n > kBM &&
                   g.ep.kind == EPI_F32 && 9 * w2 < 5 * w1) ? 1 : 0;
     }
     a.n_a = (g.a2 || a.pair) ? 2 : 1;
@@ -698,7 +687,7 @@ cudaError_t launch_gemm_tc(dflare_ctx* c, const GemmDesc& g, cudaStream_t s, std
     a.bm = kBM;
     const bool swiglu_tma = g.ep.kind == EPI_SWIGLU && (reinterpret_cast<uintptr_t>(g.ep.out) & 15u) == 0 && g.ep.ldo % 8 == 0;
     const bool f32_tma = g.ep.kind == EPI_F32 && !a.pair && (reinterpret_cast<uintptr_t>(g.ep.out) & 15u) == 0 && g.ep.ldo % 4 == 0;
-    if ((swiglu_tma || f32_tma) && g.force_splits <= 0) {
+    if (swiglu_tma || f32_tma) {
         // (every tile counts four rows more for its hand-overs: near-ties go to the taller tile. 233484 entries, d 2560: 17
         // waves of 96 rows against 25 of 64, 60 tokens 195.4 / 239.6 us, 15 tokens 180.3 / 180.5)
         long long best_cost = 0;
@@ -750,7 +739,6 @@ cudaError_t launch_gemm_tc(dflare_ctx* c, const GemmDesc& g, cudaStream_t s, std
     const int misc_bytes = 16;
     // (128-row operand reads that start at a shorter tile end inside the allocation)
     const int slack = (kBM - a.bm) * kBK * 2;
-    const int budget = g.max_smem > 0 ? std::min(g.max_smem, kSmemLimit) : kSmemLimit;
     auto epi_of = [&](int slots) {
         return a.out_mode == OUT_REGS ? a.n_a * kChunk * 128 * 4 : 4 * slots * ch * (a.out_mode == OUT_SWIGLU ? 64 : 128);
     };
@@ -759,22 +747,17 @@ cudaError_t launch_gemm_tc(dflare_ctx* c, const GemmDesc& g, cudaStream_t s, std
     // 64 -> 32: 144 tokens, d 4096: O 12.7 -> 11.1 us, down 22.9 -> 21.8; 155 logit rows of 40000 entries 74.2 -> 68.3.
     // (Where the ring stays the same, 32 cost up to 0.5 us: Q/K/V at 160 tokens 13.3 -> 13.7.)
     a.n_slots = std::min(a.bn / ch, 64 / ch);
-    if (6 * kb_bytes > budget - fixed_of(a.n_slots) && 6 * kb_bytes <= budget - fixed_of(32 / ch)) a.n_slots = 32 / ch;
+    if (6 * kb_bytes > kSmemLimit - fixed_of(a.n_slots) && 6 * kb_bytes <= kSmemLimit - fixed_of(32 / ch)) a.n_slots = 32 / ch;
     const int epi_bytes = epi_of(a.n_slots), fixed = fixed_of(a.n_slots);
     a.epi_bytes = epi_bytes;
-    if (g.kbs > 0) {
-        a.kbs = g.kbs;
-    } else {
-        // a hand-off costs about 300 clocks whatever its bytes, and a ring of two stages runs dry: four
-        // 64-wide k-blocks a stage where three stages fit, else two where three fit, else one. Measured (us
-        // after the dependency at 4 / 2 / 1): 64 tokens, d 4096: Q/K/V 11.7 / 11.5 / 12.4, down 20.0 / 19.1 / 21.0; 96
-        // tokens Q/K/V - / 11.9 / 12.8, down - / 20.1 / 22.0, LM head of 40000 entries - / 59.4 / 72.4; 16 tokens, d 2560:
-        // O 5.8 / 6.2 / 7.3. Gate/up at 2 / 1: 16 tokens, d 4096, ffn 16384 41.6 / 43.9, d 2560, ffn 19456 30.5 / 31.7; 32
-        // tokens 31.6 / 33.3; 64 tokens, d 4096, ffn 12288 34.4 / 35.1, d 2880, ffn 11520 23.6 / 24.3; 96 tokens, d 2560,
-        // ffn 9728 19.8 / 22.0.
-        a.kbs = 3 * 4 * kb_bytes <= budget - fixed ? 4 : 3 * 2 * kb_bytes <= budget - fixed ? 2 : 1;
-    }
-    if (g.force_splits > 0) best = std::min(g.force_splits, a.k_blocks);
+    // a hand-off costs about 300 clocks whatever its bytes, and a ring of two stages runs dry: four
+    // 64-wide k-blocks a stage where three stages fit, else two where three fit, else one. Measured (us
+    // after the dependency at 4 / 2 / 1): 64 tokens, d 4096: Q/K/V 11.7 / 11.5 / 12.4, down 20.0 / 19.1 / 21.0; 96
+    // tokens Q/K/V - / 11.9 / 12.8, down - / 20.1 / 22.0, LM head of 40000 entries - / 59.4 / 72.4; 16 tokens, d 2560:
+    // O 5.8 / 6.2 / 7.3. Gate/up at 2 / 1: 16 tokens, d 4096, ffn 16384 41.6 / 43.9, d 2560, ffn 19456 30.5 / 31.7; 32
+    // tokens 31.6 / 33.3; 64 tokens, d 4096, ffn 12288 34.4 / 35.1, d 2880, ffn 11520 23.6 / 24.3; 96 tokens, d 2560,
+    // ffn 9728 19.8 / 22.0.
+    a.kbs = 3 * 4 * kb_bytes <= kSmemLimit - fixed ? 4 : 3 * 2 * kb_bytes <= kSmemLimit - fixed ? 2 : 1;
     a.kb_per_split = (a.k_blocks + best - 1) / best;
     // (split ranges are not rounded to whole stages: the producer issues a partial last stage,
     // and balanced ranges beat 512-byte-aligned ones, e.g. Q/K^d/V^d 14/14/12 k-blocks rather
@@ -788,8 +771,7 @@ cudaError_t launch_gemm_tc(dflare_ctx* c, const GemmDesc& g, cudaStream_t s, std
     a.b_bytes = (uint32_t)a.bn * kBK * 2;
     a.a_bytes = (uint32_t)a.bm * kBK * 2;
     a.stage_bytes = (uint32_t)a.kbs * (a.a_bytes * a.n_a + a.b_bytes);
-    a.evict_first = g.evict_first >= 0 ? 1 : 0;
-    a.stages = std::min(kMaxStages, (budget - fixed) / (int)a.stage_bytes);
+    a.stages = std::min(kMaxStages, (kSmemLimit - fixed) / (int)a.stage_bytes);
     if (a.stages < 2) {
         if (why) *why = "tcgen05 GEMM: tile does not fit in shared memory";
         return cudaErrorInvalidValue;

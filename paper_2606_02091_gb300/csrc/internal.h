@@ -70,11 +70,6 @@ struct GemmDesc {
                            // blocks, b_group_rows rows apart, and contraction index kk reads
                            // block kk / b_kgroup at column kk % b_kgroup
     EpiParams ep;
-    int kbs = 0;           // tcgen05 GEMM: 64-wide k-blocks per pipeline stage (0 = default)
-    int max_smem = 0;      // tcgen05 GEMM: shared-memory budget per CTA in bytes (0 = default)
-    int evict_first = 0;   // tcgen05 GEMM: weights with an L2 evict-first policy (0 = yes, -1 = no)
-    int force_splits = 0;  // tcgen05 GEMM: K splits (0 = chosen from the wave count)
-    int force_bn = 0;      // two-SM GEMM: features per tile (0 = chosen from the cost model)
 };
 
 }  // namespace dfl
