@@ -666,8 +666,11 @@ cudaError_t launch_gemm_tc(dflare_ctx* c, const GemmDesc& g, cudaStream_t s, std
     // rows the pair fills all 512 TMEM columns, so a unit's epilogue no longer overlaps the next
     // unit's MMAs: pairs pay only for the cheap fp32-logit epilogue (the LM head), and only when
     // their wave count times ~1.8 single-tile units beats the single tiles' wave count (batch-16
-    // step 1.965 -> 1.947 ms). The two-SM GEMM has taken these launches over except for vocabularies
-    // whose rows do not start on 16 bytes.
+    // step 1.965 -> 1.947 ms). The two-SM GEMM has taken heads of more than 160 rows over; pairs remain for large
+    // heads of 113 to 160 rows and for vocabularies whose rows do not start on 16 bytes. Measured at 120 / 135 /
+    // 150 rows of 151936 entries, d 4096 (us): pairs 207 / 219 / 224, single tiles of 64 to 128 rows 207 / 210 / 219,
+    // two-SM 220 / 221 / 223; 120 / 150 rows of 201088 entries, d 2880: 213 / 246, 221 / 244, 222 / 226; 120 rows of
+    // 32000 entries, d 2560: 34 / 32 / 37. None of the three leads throughout.
     {
         const long long u1 = (long long)g.groups * ((g.n + kBM - 1) / kBM) * ((g.m_tok + a.bn - 1) / a.bn);
         const long long u2 = (long long)g.groups * ((g.n + 2 * kBM - 1) / (2 * kBM)) * ((g.m_tok + a.bn - 1) / a.bn);

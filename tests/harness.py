@@ -46,8 +46,7 @@ MULTI_TILE = synth.Workload(
 # (D 10), 128 query rows per KV head (G 8: two 64-row query tiles), a single fused target layer
 # with block 1 (no mask rows: nothing is drafted), and block 2
 # A ragged context fill: one call fills 700, 3 and 40 positions, so 5 of the 9 256-row token
-# tiles of the context K/V projection hold no appended row (skipped); the LM head's 500 rows end
-# inside the first tile of its second 256-row weight pair.
+# tiles of the context K/V projection hold no appended row (skipped).
 RAGGED = synth.Workload(
     "ragged_fill_bf16",
     synth.Shape(d=384, n_draft_layers=2, n_target_layers=3, n_q_heads=4, n_kv_heads=2,
@@ -60,14 +59,19 @@ LONG_FILL = synth.Workload(
     synth.Shape(d=256, n_draft_layers=2, n_target_layers=2, n_q_heads=8, n_kv_heads=4,
                 head_dim=128, ffn=256, vocab=300, block=4),
     (4000, 1200), 0.8, seed=23)
-# 240 LM-head rows (batch 16 x 15 mask positions) over a vocabulary of 297 weight tiles: the LM
-# head pairs them (149 pairs run in one wave, the single tiles would take two), and the last
-# pair's second tile lies past the matrix.
+# 240 LM-head rows (batch 16 x 15 mask positions) over a vocabulary of many weight tiles: the two-SM
+# GEMM's store of logits, whose last tile ends inside.
 WIDE_VOCAB = synth.Workload(
     "wide_vocab_bf16_b16",
     synth.Shape(d=256, n_draft_layers=1, n_target_layers=1, n_q_heads=4, n_kv_heads=2,
                 head_dim=64, ffn=256, vocab=38000, block=16),
     tuple(5 + (13 * b) % 29 for b in range(16)), 0.8, seed=25)
+# The single-SM GEMM's pairs of 128-row weight tiles, 297 tiles in all: the pairs run in one wave, the single
+# tiles would take two. 240 rows of a vocabulary whose rows do not start on 16 bytes, the last pair's second
+# tile past the matrix and its first one 111 rows; 120 rows of WIDE_VOCAB's.
+PAIRED_ODD = WIDE_VOCAB.with_(name="paired_vocab_37999_b16",
+                              shape=dataclasses.replace(WIDE_VOCAB.shape, vocab=37999))
+PAIRED_120 = WIDE_VOCAB.with_(name="paired_vocab_38000_b8", ctx_lens=WIDE_VOCAB.ctx_lens[:8])
 D10 = synth.Workload(
     "d10_bf16",
     synth.Shape(d=256, n_draft_layers=10, n_target_layers=2, n_q_heads=4, n_kv_heads=2,

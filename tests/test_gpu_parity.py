@@ -15,8 +15,8 @@ import pytest
 
 import oracle as O
 import synth
-from tests.harness import (BLOCK1, BLOCK2, BLOCK32, D10, G8, LONG_FILL, MULTI_TILE, QT2, RAGGED, SMALL_HD128,
-                           SMALL_HD64, TINY, WIDE_B16, WIDE_VOCAB,
+from tests.harness import (BLOCK1, BLOCK2, BLOCK32, D10, G8, LONG_FILL, MULTI_TILE, PAIRED_120, PAIRED_ODD, QT2,
+                           RAGGED, SMALL_HD128, SMALL_HD64, TINY, WIDE_B16, WIDE_VOCAB,
                            GpuSide, check_elem, check_kv, check_rows, check_tokens, f64, oracle_for,
                            rel_err, tolerance, verified_steps)
 
@@ -179,11 +179,11 @@ def test_attention_kernels_match_oracle(w, kernel):
     assert g.lib.device_error() == 0
 
 
-@pytest.mark.parametrize("w", [WIDE_B16, BLOCK32, MULTI_TILE, WIDE_VOCAB], ids=lambda w: w.name)
+@pytest.mark.parametrize("w", [WIDE_B16, BLOCK32, MULTI_TILE, WIDE_VOCAB, PAIRED_ODD, PAIRED_120], ids=lambda w: w.name)
 def test_wide_token_tiles_match_oracle(w):
     """256 token rows per projection (batch 16, the widest tcgen05 token tile), block 32, 288
-    rows (two token tiles, the second ragged), and a 240-row LM head over paired weight tiles:
-    fused context, cached K/V and the draft block against the oracle."""
+    rows (two token tiles, the second ragged), a 240-row LM head of the two-SM GEMM, and 240 and 120
+    rows over paired weight tiles: fused context, cached K/V and the draft block against the oracle."""
     g = GpuSide(w)
     o = oracle_for(w, g.W)
     fused = f64(g.fuse(w.ctx_lens))
