@@ -67,12 +67,15 @@ def test_simt_gemm_on_bf16_matches_oracle():
 
 
 # bf16 projections of more than 128 token rows (two-SM tiles of 256 rows x 64 to 256 features): one row
-# past 128 (gate/up only) with a vocabulary that no 16-byte row fits, one past the 176 of the summed
-# projections, a second 256-row tile of one row, odd counts of 64-wide k-blocks (5, 3, 17), feature
-# counts that end inside a tile, both head sizes, and fills whose token tiles are partly or all padding
+# past 128 (gate/up only) with a vocabulary that no 16-byte row fits, the summed projections (Q/K/V, O, down)
+# at their last 224 rows on the single-SM GEMM and one past them, second 256-row tiles of one row (a fill) and of 32, odd counts of
+# 64-wide k-blocks (5, 3, 17), feature counts that end inside a tile, both head sizes, and fills whose token
+# tiles are partly or all padding
 PAIR_CASES = [
     synth.Workload("pair_129", _shape(block=3, vocab=1003, ffn=192, d=320), tuple(3 + b % 5 for b in range(43)), 0.8, 41),
     synth.Workload("pair_192", _shape(block=32, vocab=1000, ffn=1088, d=320, n_q_heads=8), (40, 3, 33, 1, 17, 64), 0.8, 42),
+    synth.Workload("pair_224", _shape(block=32, vocab=1000, ffn=1088, d=320, n_q_heads=8), (40, 3, 33, 1, 17, 64, 5), 0.8, 48),
+    synth.Workload("pair_225", _shape(block=5, vocab=1000, ffn=1088, d=320, n_q_heads=8), tuple(3 + b % 7 for b in range(45)), 0.8, 49),
     synth.Workload("pair_160_odd_vocab", _shape(block=32, vocab=1003, ffn=320), (40, 3, 33, 1, 17), 0.8, 46),
     synth.Workload("pair_fill_257", _shape(head_dim=128, ffn=192), (257,), 0.8, 43),
     synth.Workload("pair_288", _shape(block=32, vocab=2004, head_dim=128, ffn=704, d=576), (300, 1, 2, 5, 257, 9, 3, 30, 64), 0.8, 44),
