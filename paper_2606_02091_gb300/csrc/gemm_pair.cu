@@ -158,8 +158,8 @@ __global__ void __launch_bounds__(kPairThreads, 1) gemm_pair_kernel(const __grid
         asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
         asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
     }
-    // a context fill of sequences with different lengths: as in the single-SM GEMM, units run over
-    // the token tiles that hold appended rows (both CTAs of a pair form the same list)
+    // a context fill of sequences with different lengths: units run over the token tiles that hold appended
+    // rows, listed in shared memory (both CTAs of a pair form the same list), not over the padding
     int* const tok_list = reinterpret_cast<int*>(misc + 4);
     if (args.compact) {
         pdl_wait();

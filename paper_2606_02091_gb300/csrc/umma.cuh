@@ -1,4 +1,5 @@
-// mbarrier, TMA and tcgen05 helpers of the projection GEMMs (sm_103a inline PTX).
+// mbarrier, TMA and tcgen05 helpers of the projection GEMMs (sm_103a inline PTX); the attention uses its thread
+// election and asynchronous tensor-memory loads, the context-fill fusion its election.
 #pragma once
 #include <cuda.h>
 
