@@ -144,7 +144,7 @@ __device__ __forceinline__ void store4(float* p, int i, int c1, bool vec, const 
 // ---------------------------------------------------------------------------------- drafting
 // Grid (chunks, rows), chunk a multiple of 8: every thread takes groups of eight logits and the
 // one Philox block that covers them. copy (when given) receives the logits as they are read.
-__global__ void __launch_bounds__(256) sample_kernel(const float* __restrict__ logits, int V, int rows,
+__global__ void __launch_bounds__(256, 4) sample_kernel(const float* __restrict__ logits, int V, int rows,
                                                      int chunk, float inv_t, uint64_t seed,
                                                      const uint64_t* __restrict__ step_dev,
                                                      unsigned long long* slot, uint32_t* cnt,
@@ -350,7 +350,7 @@ __device__ __forceinline__ void accept_block(Accept& sh, const float* target, co
 // max(0, p - q) at its first rejected position a, or from p at the last target row when every draft
 // was kept. The last CTA writes accept_len = a + 1 and the token, re-arms the slots, and advances the
 // step counter.
-__global__ void __launch_bounds__(256) spec_resample_kernel(
+__global__ void __launch_bounds__(256, 3) spec_resample_kernel(
     const float* __restrict__ target, const float* __restrict__ draft_logits,
     const int32_t* __restrict__ draft, int V, int B, int batch, int chunk, int stat_chunks, float inv_t,
     uint64_t seed, uint64_t* step_dev, const float2* __restrict__ part, int32_t* spec_a,
