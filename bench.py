@@ -309,8 +309,7 @@ def gemm_traffic(w):
         return None
     d = json.load(open(path))
     csrc = os.path.join(ROOT, "paper_2606_02091_gb300", "csrc")
-    src = open(os.path.join(csrc, "gemm_tc.cu"), "rb").read() + \
-        open(os.path.join(csrc, "epilogue.cuh"), "rb").read()
+    src = b"".join(open(os.path.join(csrc, f), "rb").read() for f in ("gemm_tc.cu", "epilogue.cuh", "umma.cuh"))
     if hashlib.sha256(src).hexdigest()[:16] != d.get("source_sha256_16"):
         return None
     return d.get("dram_bytes_per_step")

@@ -7,8 +7,8 @@
 // 128-row UMMA M dimension runs over weight rows (output features) and the small token count is
 // the UMMA N dimension (16..256), so one instruction covers a 128 x bn x 16 piece.
 //
-// Work unit = (group, 128-feature tile, token tile, K split); for an LM head over 128+ token rows,
-// a pair of adjacent 128-feature tiles (two accumulators over one activation tile). A
+// Work unit = (group, 128-feature tile, token tile, K split); for a large LM head over 113 or more token
+// rows, a pair of adjacent 128-feature tiles (two accumulators over one activation tile). A
 // persistent grid of one CTA per SM walks the units. Per CTA (192 threads):
 //   warp 4    TMA producer: per stage, kbs consecutive 128x64 bf16 weight tiles (+ the up tiles
 //             for SwiGLU) and the matching bn x 64 activation tiles, 128-byte swizzled; weights

@@ -143,7 +143,8 @@ __device__ __forceinline__ void store4(float* p, int i, int c1, bool vec, const 
 
 // ---------------------------------------------------------------------------------- drafting
 // Grid (chunks, rows), chunk a multiple of 8: every thread takes groups of eight logits and the
-// one Philox block that covers them. copy (when given) receives the logits as they are read.
+// one Philox block that covers them. copy (when given) receives the logits as they are read. (The
+// bound of four CTAs per SM is what the compiler aims at by itself, 64 registers; unsaid, it spills 16 bytes.)
 __global__ void __launch_bounds__(256, 4) sample_kernel(const float* __restrict__ logits, int V, int rows,
                                                      int chunk, float inv_t, uint64_t seed,
                                                      const uint64_t* __restrict__ step_dev,
@@ -349,7 +350,8 @@ __device__ __forceinline__ void accept_block(Accept& sh, const float* target, co
 // Grid (chunks, batch): the acceptance decisions and the replacement draw of every sequence, from
 // max(0, p - q) at its first rejected position a, or from p at the last target row when every draft
 // was kept. The last CTA writes accept_len = a + 1 and the token, re-arms the slots, and advances the
-// step counter.
+// step counter. (Likewise three CTAs, 80 registers; unsaid, 64 bytes of spill loads: verification of 4 x 16 rows
+// 42.0 -> 41.4 us.)
 __global__ void __launch_bounds__(256, 3) spec_resample_kernel(
     const float* __restrict__ target, const float* __restrict__ draft_logits,
     const int32_t* __restrict__ draft, int V, int B, int batch, int chunk, int stat_chunks, float inv_t,

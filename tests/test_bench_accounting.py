@@ -96,3 +96,23 @@ def test_launches_behind_the_fp32_attention():
     assert [bench.kernels_per_trace(s, 1, n, 152)["attention"] for n in (128, 184, 185, 4000)] == [1, 1, 2, 2]
     assert bench.kernels_per_trace(s, 152, 4000, 152)["attention"] == 1
     assert bench.kernels_per_trace(synth.preset("qwen3_4b").shape, 1, 4000, 152)["attention"] == 1
+
+
+@pytest.mark.parametrize("changed", [None, "gemm_tc.cu", "epilogue.cuh", "umma.cuh"])
+def test_gemm_traffic_belongs_to_the_sources_it_was_measured_on(tmp_path, monkeypatch, changed):
+    """The committed DRAM bytes are reported only while every source of the kernel is the one they came from."""
+    import hashlib
+    import json
+    csrc = tmp_path / "paper_2606_02091_gb300" / "csrc"
+    csrc.mkdir(parents=True)
+    (tmp_path / "profiles").mkdir()
+    files = ("gemm_tc.cu", "epilogue.cuh", "umma.cuh")
+    for f in files:
+        (csrc / f).write_text(f + "\n")
+    h = hashlib.sha256(b"".join((csrc / f).read_bytes() for f in files)).hexdigest()[:16]
+    (tmp_path / "profiles" / "gemm_tc_traffic_qwen3_4b.json").write_text(
+        json.dumps({"dram_bytes_per_step": 7.0, "source_sha256_16": h}))
+    monkeypatch.setattr(bench, "ROOT", str(tmp_path))
+    if changed:
+        (csrc / changed).write_text("other\n")
+    assert bench.gemm_traffic(synth.preset("qwen3_4b")) == (None if changed else 7.0)
