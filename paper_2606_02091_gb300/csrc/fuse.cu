@@ -238,10 +238,12 @@ __device__ __forceinline__ bool fill_wait(uint32_t bar, uint32_t parity, volatil
 
 // Waits, within one limit for all of them, for the copies of a ring of ns slots whose next stage to read is the one
 // in slot st (its full barrier's phase: `phase`). A slot that was not refilled uses the limit up.
-__device__ __noinline__ void fill_drain(uint32_t full_bar0, int ns, int st, uint32_t phase, uint32_t* err) {
+__device__ __forceinline__ void fill_drain(uint32_t full_bar0, int ns, int st, uint32_t phase, uint32_t* err) {
     atomicOr(err, DFLARE_DEVERR_TIMEOUT);
-    volatile int never = 0;
-    for (int i = 0; i < ns; ++i) fill_wait(full_bar0 + 8u * i, i >= st ? phase : phase ^ 1u, &never);
+    const uint64_t t0 = globaltimer_ns();
+    for (int i = 0; i < ns; ++i)
+        while (!fill_try(full_bar0 + 8u * i, i >= st ? phase : phase ^ 1u) && globaltimer_ns() - t0 < kFillWaitNs) {
+        }
 }
 
 // Two fp32 lanes in one 64-bit register: the fill's sums use the paired FMA (fma.rn.f32x2, each
