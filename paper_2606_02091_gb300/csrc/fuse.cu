@@ -187,20 +187,25 @@ __global__ void __launch_bounds__(256) fuse_layers_kernel(
 
 // Many positions (context fill): a persistent grid of one or two CTAs per SM walks the positions
 // (no cluster). The T target rows of each position (d contiguous elements each) stream through a ring of
-// `ns` shared-memory stages of kRB rows as 1-D bulk copies, the stage sequence running on across
+// `ns` shared-memory stages of a few rows as 1-D bulk copies, the stage sequence running on across
 // positions. Each stage has a "full" mbarrier (the copies landed) and an "empty" one that every warp
-// arrives on once it has read the stage; the warps take turns at refilling a slot, so no warp exists only
-// to copy: with one, an SM sub-partition holds a warp more and every thread a fifth fewer registers, and
-// the 128 sums of eight draft layers did not fit. Thread t forms the D (<= DMAX) draft-layer sums of 8
-// features (D <= 5) or two groups of 8 (more: half the reads of the weights alpha per sum, which at one
-// group cost as many shared-memory clocks as the rows) in registers; at the end of a position the D sums
-// of squares take 9 shuffles and one named barrier. Every wait is bounded; a CTA that times out sets
-// DFLARE_DEVERR_TIMEOUT and stops.
+// arrives on once it has read the stage. Thread t forms the D (<= DMAX) draft-layer sums of 8 features or
+// (NF 2) two groups of 8 in registers; at the end of a position the D sums of squares take 9 shuffles and one
+// named barrier. Every wait is bounded; a CTA that times out sets DFLARE_DEVERR_TIMEOUT and stops.
+// Who refills the ring:
+// - The warps take turns (PROD false), for many target rows of many features: a warp that only copies would
+//   cost every thread a fifth of its registers, and with two feature groups (D 6 to 8: half the reads of the
+//   weights alpha per sum, which at one group cost as many shared-memory clocks as the rows) the 128 sums of
+//   eight draft layers did not fit beside it.
+// - A producer warp (PROD), for few rows or few features: there a position takes a few hundred clocks, the others
+//   wait at its barrier for the warp whose turn it is, and a CTA of few warps has registers to spare.
 // Bound by HBM for up to four draft layers, by the fp32 FMAs above (10.4k of 20k clocks a position at D 8,
-// d 4096). Measured, target rows read + fused rows written per second against a producer warp, one group
-// and three barriers a position: d 4096 D 8 4.0 -> 4.8 TB/s, D 4 5.5 -> 6.3, D 2 5.5 -> 6.2; d 2560 D 5
-// (2048 positions) 4.3 -> 4.7. Stages of 3 / 4 / 6 / 9 rows at D 8: 679 / 652 / 631 / 827 us for 8192 positions;
-// refilling one stage behind instead of two 631 -> 615.
+// d 4096). Measured, T 36, target rows read + fused rows written per second, by turns against an earlier form with
+// a producer warp, one group and three barriers a position: d 4096 D 8 4.0 -> 4.8 TB/s, D 4 5.5 -> 6.3, D 2
+// 5.5 -> 6.2; d 2560 D 5 (2048 positions) 4.3 -> 4.7. Stages of 3 / 4 / 6 / 9 rows at D 8: 679 / 652 / 631 / 827 us
+// for 8192 positions; refilling one stage behind instead of two 631 -> 615. 2048 positions (us), the earlier form /
+// by turns / with the producer warp: d 1024 D 8 T 8 47 / 67 / 45, d 512 D 6 T 12 56 / 61 / 41, d 256 D 1 T 36
+// 40 / 45 / 30, d 4096 D 2 T 4 39 / 43 / 40, fp32 d 512 D 2 T 8 21 / 27 / 21.
 constexpr int kLag = 1;         // stages between a slot's use and its refill
 constexpr int kMaxNS = 16;      // most stages in the ring
 constexpr int kMinNS = 3;
@@ -277,15 +282,18 @@ __device__ __forceinline__ void load8x2(const float* p, f32x2* h) {
     h[3] = pk2(b.z, b.w);
 }
 
+// target rows per stage, and up to how many a producer warp refills the ring whatever the features (see fuse_layers_t)
+template <class T, bool PROD>
+constexpr int kRowsPerStage = sizeof(T) == 2 ? 6 : PROD ? 4 : 3;
 template <class T>
-constexpr int kRowsPerStage = sizeof(T) == 2 ? 6 : 3;   // target rows
+constexpr int kFewRows = sizeof(T) == 2 ? 8 : 4;
 
-template <class T, int DMAX, int NF>
+template <class T, int DMAX, int NF, bool PROD>
 __device__ __forceinline__ void fuse_rows_body(
     const T* __restrict__ H, const float* __restrict__ alpha, const T* __restrict__ gain,
     T* __restrict__ F, T* __restrict__ F_out, const int32_t* __restrict__ app_cnt, int D, int Tn,
     int batch, int n_max, int d, long long f_layer_rows, float eps, int ns, uint32_t* err) {
-    constexpr int kRB = kRowsPerStage<T>;
+    constexpr int kRB = kRowsPerStage<T, PROD>;
     pdl_trigger();
     extern __shared__ __align__(128) uint8_t stage_mem[];   // [ns][kRB][d]
     constexpr int DP = (DMAX + 1) & ~1;                       // DMAX rounded up to even
@@ -295,7 +303,7 @@ __device__ __forceinline__ void fuse_rows_body(
     __shared__ __align__(8) uint64_t full_bar[kMaxNS], empty_bar[kMaxNS];
     __shared__ int abort_flag;
     const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
-    const int n_cw = (int)(blockDim.x >> 5), n_ct = (int)blockDim.x;
+    const int n_cw = (int)(blockDim.x >> 5) - (PROD ? 1 : 0), n_ct = PROD ? n_cw * 32 : (int)blockDim.x;   // that form sums
     const uint32_t fb0 = (uint32_t)__cvta_generic_to_shared(&full_bar[0]);
     const uint32_t eb0 = (uint32_t)__cvta_generic_to_shared(&empty_bar[0]);
     const uint32_t sbase = (uint32_t)__cvta_generic_to_shared(stage_mem);
@@ -330,7 +338,7 @@ __device__ __forceinline__ void fuse_rows_body(
     int first = (int)blockIdx.x;
     if (first < n_pos && !valid(first)) first = next_pos(first);
 
-    // The stages run on across positions. Stage g goes into slot g % ns; the ring is filled once at the
+    // The stages run on across positions. Stage g goes into slot g % ns. By turns: the ring is filled once at the
     // start, then each step's refill is issued by one elected thread, warp g % n_cw at its step g, into
     // the slot of stage g - kLag, which the other warps have left by then as a rule. (ppid, pk): the
     // next stage to issue, tracked by every thread.
@@ -353,10 +361,30 @@ __device__ __forceinline__ void fuse_rows_body(
                 "l"(H + (size_t)(j0 + u) * lstride + (size_t)ppid * d), "r"(row_bytes), "r"(bar)
                 : "memory");
     };
-    for (int i = 0; i < ns && ppid < n_pos; ++i, next_stage())
-        if (warp == 0 && elect_one()) issue(i);
+    if constexpr (!PROD)
+        for (int i = 0; i < ns && ppid < n_pos; ++i, next_stage())
+            if (warp == 0 && elect_one()) issue(i);
 
-    {
+    if (PROD && warp == n_cw) {
+        if (elect_one()) {
+            int st = 0;
+            uint32_t phase = 0;
+            bool ok = true;
+            for (; ppid < n_pos; next_stage()) {
+                if (!fill_wait(eb0 + 8u * st, phase ^ 1u, abrt)) {
+                    ok = false;
+                    break;
+                }
+                issue(st);
+                if (++st == ns) {
+                    st = 0;
+                    phase ^= 1u;
+                }
+            }
+            // after a timeout: the last copies of every slot land before the CTA leaves
+            if (!ok) fill_drain(fb0, ns, st, phase ^ 1u, err);
+        }
+    } else {
         // thread t owns NF groups of 8 features, n_ct groups apart; a thread without its last group reads
         // group 0 instead and drops the result
         int e[NF], er[NF];
@@ -418,7 +446,7 @@ __device__ __forceinline__ void fuse_rows_body(
                     add_stage(std::integral_constant<int, NF - 1>{});
                 __syncwarp();
                 if (lane == 0) asm volatile("mbarrier.arrive.shared::cta.b64 _, [%0];" ::"r"(eb0 + 8u * st) : "memory");
-                if (rst >= 0 && ppid < n_pos) {
+                if (!PROD && rst >= 0 && ppid < n_pos) {
                     if (warp == turn && elect_one()) {
                         if (fill_wait(eb0 + 8u * rst, rphase, abrt))
                             issue(rst);
@@ -537,11 +565,15 @@ __device__ __forceinline__ void fuse_rows_body(
 #define FUSE_ROWS_ARGS H, alpha, gain, F, F_out, app_cnt, D, Tn, batch, n_max, d, f_layer_rows, eps, ns, err
 template <class T, int DMAX, int NF>
 __global__ void __launch_bounds__(512 / NF, 1) fuse_rows_kernel(FUSE_ROWS_PARAMS) {
-    fuse_rows_body<T, DMAX, NF>(FUSE_ROWS_ARGS);
+    fuse_rows_body<T, DMAX, NF, false>(FUSE_ROWS_ARGS);
 }
 template <class T, int DMAX>
 __global__ void __launch_bounds__(320, 2) fuse_rows2_kernel(FUSE_ROWS_PARAMS) {
-    fuse_rows_body<T, DMAX, 1>(FUSE_ROWS_ARGS);
+    fuse_rows_body<T, DMAX, 1, false>(FUSE_ROWS_ARGS);
+}
+template <class T, int DMAX, int THREADS, int PER_SM>
+__global__ void __launch_bounds__(THREADS + 32, PER_SM) fuse_rows_prod_kernel(FUSE_ROWS_PARAMS) {
+    fuse_rows_body<T, DMAX, 1, true>(FUSE_ROWS_ARGS);
 }
 #undef FUSE_ROWS_PARAMS
 #undef FUSE_ROWS_ARGS
@@ -557,30 +589,38 @@ cudaError_t fuse_layers_t(dflare_ctx* c, const void* hidden, int n_max, void* fu
     const T* gain = static_cast<const T*>(c->w.fuse_norm);
     T* F = static_cast<T*>(c->fused);
     T* Fo = static_cast<T*>(fused_out);
-    // context fill: CTAs of d / 8 threads (up to five draft layers) or d / 16 (six to eight, at least enough
-    // warps for a balanced SM), two per SM when their registers allow (rings of about 100 KB), else one
-    // (about 200 KB); at most kMaxNS stages
-    const size_t stage_bytes = (size_t)kRowsPerStage<T> * g.d * sizeof(T);
-    const int Dn = g.n_draft_layers, nf = Dn <= 5 ? 1 : 2;
-    const int threads = std::min(512 / nf, (g.d / 8 + 31) / 32 * 32);   // (d <= 4096)
+    // Context fill: CTAs of d / 8 threads, or of d / 16 where six to eight draft layers take two feature groups per
+    // thread, two per SM when their registers allow (rings of about 100 KB), else one (about 200 KB); at most kMaxNS
+    // stages. A producer warp refills the ring up to 1024 features, or 2048 at six to eight draft layers (where its
+    // CTA has registers for one group's sums), and for up to kFewRows target rows. Across those lines, 2048 positions,
+    // by turns / producer warp (us): d 1024 D 4 T 36 45.2 / 42.9, d 1536 D 2 T 24
+    // 10 % behind with the producer warp, d 2048 D 4 T 8 33.6 / 31.6, d 2048 D 6 T 36 121.7 / 102.4, fp32 d 1024 D 2
+    // T 12 31.6 / 31.6.
+    const int Dn = g.n_draft_layers, nf = Dn <= 5 ? 1 : 2, d_threads = (g.d / 8 + 31) / 32 * 32;   // (d <= 4096)
+    const bool prod = Dn > 5 ? g.d <= 2048 : g.d <= 1024 || (g.n_target_layers <= kFewRows<T> && (Dn < 5 || g.d <= 2048));
+    const size_t stage_bytes = (size_t)(prod ? kRowsPerStage<T, true> : kRowsPerStage<T, false>) * g.d * sizeof(T);
     if ((long long)c->batch * n_max >= 2LL * c->num_sms && Dn <= 8 && g.n_target_layers <= 64 &&
         kMinNS * stage_bytes <= kRingBytes) {
         static PerDeviceOnce rconf;
         const cudaError_t re = rconf([] {
             for (auto k : {fuse_rows_kernel<T, 4, 1>, fuse_rows_kernel<T, 5, 1>, fuse_rows_kernel<T, 8, 2>,
-                           fuse_rows2_kernel<T, 4>, fuse_rows2_kernel<T, 5>}) {
+                           fuse_rows2_kernel<T, 4>, fuse_rows2_kernel<T, 5>, fuse_rows_prod_kernel<T, 4, 512, 1>,
+                           fuse_rows_prod_kernel<T, 5, 256, 2>, fuse_rows_prod_kernel<T, 8, 256, 1>}) {
                 cudaError_t e = cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kRingBytes);
                 if (e != cudaSuccess) return e;
             }
             return cudaSuccess;
         });
         if (re != cudaSuccess) return re;
-        auto rk = Dn <= 4 ? fuse_rows_kernel<T, 4, 1> : Dn == 5 ? fuse_rows_kernel<T, 5, 1> : fuse_rows_kernel<T, 8, 2>;
-        auto rk2 = Dn <= 4 ? fuse_rows2_kernel<T, 4> : fuse_rows2_kernel<T, 5>;   // (D <= 5 below)
         int ns = (int)std::min<size_t>(kMaxNS, kRingBytes / stage_bytes), per_sm = 1;
         const int ns2 = (int)std::min<size_t>(kMaxNS, kRingBytes / 2 / stage_bytes);
+        auto rk = prod ? (Dn > 5 ? fuse_rows_prod_kernel<T, 8, 256, 1>
+                          : d_threads <= 256 ? fuse_rows_prod_kernel<T, 5, 256, 2> : fuse_rows_prod_kernel<T, 4, 512, 1>)
+                  : Dn <= 4 ? fuse_rows_kernel<T, 4, 1> : Dn == 5 ? fuse_rows_kernel<T, 5, 1> : fuse_rows_kernel<T, 8, 2>;
+        auto rk2 = prod ? fuse_rows_prod_kernel<T, 5, 256, 2> : Dn <= 4 ? fuse_rows2_kernel<T, 4> : fuse_rows2_kernel<T, 5>;
+        const int threads = prod ? d_threads + 32 : std::min(512 / nf, d_threads);
         int fit = 0;
-        if (threads <= 320 && Dn <= 5 && ns2 >= kMinNS &&
+        if (Dn <= 5 && ns2 >= kMinNS && d_threads <= (prod ? 256 : 320) &&
             cudaOccupancyMaxActiveBlocksPerMultiprocessor(&fit, rk2, threads, (size_t)ns2 * stage_bytes) ==
                 cudaSuccess && fit >= 2) {
             rk = rk2;

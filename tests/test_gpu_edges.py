@@ -151,15 +151,28 @@ def test_logit_tiles_match_oracle(w):
     _step_matches_oracle(w)
 
 
-# context fills of at least two positions per SM: one and two feature groups per thread (five and six draft
-# layers), two CTAs per SM, warps with and without their second group, target-layer counts that end inside
-# a stage of 6 (bf16) or 3 (fp32) rows, fewer target rows than a stage, positions past a sequence's end
+# context fills of at least two positions per SM. The ring refilled by the warps in turn: one and two feature groups
+# per thread (five and six draft layers), two CTAs per SM, warps with and without their second group; by a
+# producer warp: one and two CTAs per SM, the widest rows of each, one feature past the narrow ones. Target-layer
+# counts that end inside a stage of 6 (bf16) or 3 and 4 (fp32) rows, fewer target rows than a stage, positions past
+# a sequence's end, one position per step of the grid
 FILL_CASES = [
     synth.Workload("fill_d2112_D6_T7", _shape(d=2112, n_draft_layers=6, n_target_layers=7, ffn=64, block=2), (170, 140), 0.8, 51),
     synth.Workload("fill_d4096_D8_T3", _shape(d=4096, n_draft_layers=8, n_target_layers=3, ffn=64, block=2), (305,), 0.8, 52),
     synth.Workload("fill_d704_D5_T13", _shape(d=704, n_draft_layers=5, n_target_layers=13, ffn=64, block=2), (300, 9), 0.8, 53),
     synth.Workload("fill_d2816_D3_T6", _shape(d=2816, n_draft_layers=3, n_target_layers=6, ffn=64, block=2), (305,), 0.8, 54),
     synth.Workload("fill_f32_d320_D7_T5", _shape(dtype="f32", d=320, n_draft_layers=7, n_target_layers=5, ffn=64, block=2), (306,), 0.8, 55),
+    synth.Workload("fill_d1088_D5_T13", _shape(d=1088, n_draft_layers=5, n_target_layers=13, ffn=64, block=2), (300, 9), 0.8, 56),
+    synth.Workload("fill_d2816_D3_T9", _shape(d=2816, n_draft_layers=3, n_target_layers=9, ffn=64, block=2), (305,), 0.8, 57),
+    synth.Workload("fill_d2048_D8_T8", _shape(d=2048, n_draft_layers=8, n_target_layers=8, ffn=64, block=2), (170, 1, 140), 0.8, 58),
+    synth.Workload("fill_d1024_D1_T1", _shape(d=1024, n_draft_layers=1, n_target_layers=1, ffn=64, block=2), (700,), 0.8, 59),
+    synth.Workload("fill_d64_D5_T36", _shape(d=64, n_draft_layers=5, n_target_layers=36, ffn=64, block=2), (160, 3, 150), 0.8, 60),
+    synth.Workload("fill_d2048_D5_T8", _shape(d=2048, n_draft_layers=5, n_target_layers=8, ffn=64, block=2), (305,), 0.8, 74),
+    synth.Workload("fill_d4096_D4_T8", _shape(d=4096, n_draft_layers=4, n_target_layers=8, ffn=64, block=2), (305,), 0.8, 75),
+    synth.Workload("fill_f32_d2112_D6_T7", _shape(dtype="f32", d=2112, n_draft_layers=6, n_target_layers=7, ffn=64, block=2), (170, 140), 0.8, 76),
+    synth.Workload("fill_f32_d1088_D2_T5", _shape(dtype="f32", d=1088, n_draft_layers=2, n_target_layers=5, ffn=64, block=2), (305,), 0.8, 77),
+    synth.Workload("fill_f32_d1024_D5_T9", _shape(dtype="f32", d=1024, n_draft_layers=5, n_target_layers=9, ffn=64, block=2), (300, 9), 0.8, 78),
+    synth.Workload("fill_f32_d4096_D2_T4", _shape(dtype="f32", d=4096, n_draft_layers=2, n_target_layers=4, ffn=64, block=2), (305,), 0.8, 79),
 ]
 
 
