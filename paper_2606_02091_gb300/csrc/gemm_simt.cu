@@ -8,8 +8,8 @@
 // tokens), and the 32 lanes' sums are added in a butterfly that halves the values a lane holds at
 // each step. No shared memory and no barrier until the epilogue, the first weights are loaded
 // before the dependency wait, and a lane's serial chain is K / 32 FMAs per sum. Each 16-byte load
-// feeds 16 (weights: 4 TT) FMAs, so the same form also runs a fill of hundreds of tokens near the
-// L1 limit. The earlier form (128 rows x 16 tokens per CTA, K in shared-memory chunks of 16 between
+// feeds 16 (weights: 4 TT) FMAs; projections of many token rows take the tiled form below. The
+// earlier form (128 rows x 16 tokens per CTA, K in shared-memory chunks of 16 between
 // two barriers) waited a memory round trip per chunk (ncu: 32 us at K 256, 92 us at K 768). With this
 // kernel and the fp32 attention of attention.cu the first step of a 128-position sequence on the fp32
 // drafter (d 256, 4 layers, block 8) went from 968 to 158 us, and to 134 with two chunks of K per round.
@@ -135,12 +135,146 @@ __global__ void __launch_bounds__(kSimtThreads) gemm_simt_kernel(
     }
 }
 
+// Many token rows: one CTA computes 128 weight rows x 64 tokens (SwiGLU: 128 of gate, the same 128 of up x 32
+// tokens), 8 x 4 sums (2 x 8 x 2) per thread, K in chunks of 16 through two shared-memory buffers, the next
+// chunk's loads in flight behind the FMAs. The warp-per-rows form, whose eight warps each load the tokens for
+// themselves, had fallen behind the one before it here: fp32 (us, the one before / warp per rows / tiles), 16384 rows
+// x 512 x 1024 1180 / 1389 / 508, 32768 x 512 x 512 1175 / 1538 / 532, 8192 x 256 x 256 96 / 105 / 47. Bound by the
+// FMAs and the shared-memory reads that feed them.
+// A thread adds a chunk's products in two chains of 8, four chunks' sums to a partial sum and that to the total:
+// the error against 64 bits is that of the warp-per-rows form at K 256 (8.1e-8 of the result's rms) and below it
+// beyond (K 2048 1.2e-7 / 1.6e-7; chains of 64 would have 1.5e-7 at K 256).
+constexpr int kTileK = 16, kFlush = 4;
+template <class T, bool DUAL>
+__global__ void __launch_bounds__(kSimtThreads) gemm_simt_tiled_kernel(
+    const T* __restrict__ A, const T* __restrict__ A2, const T* __restrict__ Bm, int n, int k, int m_tok,
+    long long a_group_rows, long long b_group_rows, int b_shared, int b_kgroup, int n_tiles, EpiParams ep) {
+    constexpr int NA = DUAL ? 2 : 1, TOK = 64 / NA, TPT = TOK / 16;   // tokens per CTA and thread
+    constexpr int LDA = 128 + 4, LDB = TOK + 4;
+    constexpr int OPS = 2 * kTileK * (NA * LDA + LDB), TILES = NA * TOK * 128;
+    __shared__ __align__(16) float buf[OPS > TILES ? OPS : TILES];   // operands, then the epilogue's tiles
+    pdl_wait();
+    pdl_trigger();   // after the wait: see gemm_tc_kernel
+    const int n_tile = blockIdx.x % n_tiles, group = blockIdx.x / n_tiles, tok0 = blockIdx.y * TOK;
+    const int tid = threadIdx.x, tx = tid & 15, ty = tid >> 4;
+    const T* Bg = Bm + (size_t)(b_shared || b_kgroup > 0 ? 0 : group) * b_group_rows * k;
+    const size_t b_ld = b_kgroup > 0 ? b_kgroup : k;
+    const int lr = tid >> 2, lk = (tid & 3) * 4;    // this thread's row (+ 64) and k of a chunk's loads
+    const T* ap[NA][2];
+#pragma unroll
+    for (int a = 0; a < NA; ++a)
+#pragma unroll
+        for (int h = 0; h < 2; ++h)
+            ap[a][h] = (a ? A2 : A) + ((size_t)group * a_group_rows + min(n_tile * 128 + lr + 64 * h, n - 1)) * k + lk;
+    const bool lb = lr < TOK;
+    const T* const bp = Bg + (size_t)min(tok0 + (lb ? lr : 0), m_tok - 1) * b_ld + lk;   // rows past the end: not stored
+    auto b_at = [&](int k0) {   // contraction over stacked activation groups (Eq. 1): a chunk lies in one
+        if (b_kgroup <= 0) return bp + k0;
+        const int z = k0 / b_kgroup;
+        return bp + (size_t)z * b_group_rows * b_kgroup + (k0 - z * b_kgroup);
+    };
+    auto As = [&](int st, int a) { return buf + (st * NA + a) * kTileK * LDA; };
+    auto Bs = [&](int st) { return buf + 2 * NA * kTileK * LDA + st * kTileK * LDB; };
+    float4 ra[NA][2], rb = make_float4(0.f, 0.f, 0.f, 0.f);
+    auto load = [&](int k0) {
+#pragma unroll
+        for (int a = 0; a < NA; ++a)
+#pragma unroll
+            for (int h = 0; h < 2; ++h) ra[a][h] = ld4(ap[a][h] + k0);
+        if (lb) rb = ld4(b_at(k0));
+    };
+    auto put = [&](float* d, int ld, float4 v) {
+        d[0] = v.x;
+        d[ld] = v.y;
+        d[2 * ld] = v.z;
+        d[3 * ld] = v.w;
+    };
+    auto store = [&](int st) {
+#pragma unroll
+        for (int a = 0; a < NA; ++a)
+#pragma unroll
+            for (int h = 0; h < 2; ++h) put(As(st, a) + lk * LDA + lr + 64 * h, LDA, ra[a][h]);
+        if (lb) put(Bs(st) + lk * LDB + lr, LDB, rb);
+    };
+    constexpr int S = NA * 8 * TPT;                 // sums of a thread, [accumulator][feature][token]
+    float acc[S], part[S];
+#pragma unroll
+    for (int i = 0; i < S; ++i) acc[i] = part[i] = 0.f;
+    load(0);
+    store(0);
+    __syncthreads();
+    const int chunks = k / kTileK;   // (k is a multiple of 64)
+    for (int c = 0; c < chunks; ++c) {
+        const int st = c & 1;
+        if (c + 1 < chunks) load((c + 1) * kTileK);
+        float sum[2][S];
+#pragma unroll
+        for (int h = 0; h < 2; ++h) {
+#pragma unroll
+            for (int i = 0; i < S; ++i) sum[h][i] = 0.f;
+#pragma unroll
+            for (int kk = h * 8; kk < h * 8 + 8; ++kk) {
+                float b[TPT];
+#pragma unroll
+                for (int t = 0; t < TPT; ++t) b[t] = Bs(st)[kk * LDB + ty * TPT + t];
+#pragma unroll
+                for (int a = 0; a < NA; ++a) {
+                    const float4 lo = *reinterpret_cast<const float4*>(As(st, a) + kk * LDA + tx * 4);
+                    const float4 hi = *reinterpret_cast<const float4*>(As(st, a) + kk * LDA + 64 + tx * 4);
+                    const float w[8] = {lo.x, lo.y, lo.z, lo.w, hi.x, hi.y, hi.z, hi.w};
+#pragma unroll
+                    for (int f = 0; f < 8; ++f)
+#pragma unroll
+                        for (int t = 0; t < TPT; ++t) {
+                            float& x = sum[h][(a * 8 + f) * TPT + t];
+                            x = fmaf(w[f], b[t], x);
+                        }
+                }
+            }
+        }
+#pragma unroll
+        for (int i = 0; i < S; ++i) part[i] += sum[0][i] + sum[1][i];
+        if (c % kFlush == kFlush - 1) {
+#pragma unroll
+            for (int i = 0; i < S; ++i) {
+                acc[i] += part[i];
+                part[i] = 0.f;
+            }
+        }
+        if (c + 1 < chunks) store(st ^ 1);   // (read two chunks ago, before the last barrier)
+        __syncthreads();
+    }
+    // the epilogue's tiles [16-token chunk][accumulator][token][feature]
+#pragma unroll
+    for (int a = 0; a < NA; ++a)
+#pragma unroll
+        for (int t = 0; t < TPT; ++t) {
+            const int tok = ty * TPT + t;
+            float* d = buf + (((tok >> 4) * NA + a) * kEpiChunk + (tok & 15)) * 128 + tx * 4;
+            const float* v = acc + a * 8 * TPT + t;
+            *reinterpret_cast<float4*>(d) = make_float4(v[0], v[TPT], v[2 * TPT], v[3 * TPT]);
+            *reinterpret_cast<float4*>(d + 64) = make_float4(v[4 * TPT], v[5 * TPT], v[6 * TPT], v[7 * TPT]);
+        }
+    __syncthreads();
+    for (int ch = tid >> 7; ch < TOK / kEpiChunk; ch += 2)
+        apply_epilogue<T>(ep, buf + ch * NA * kEpiChunk * 128, group, n_tile, tok0 + ch * kEpiChunk, tid & 127);
+}
+
 template <class T>
 cudaError_t launch_t(dflare_ctx* c, const GemmDesc& g, cudaStream_t s) {
-    const int per = g.a2 ? 16 : kRows;
-    const int n_slices = (g.n + per - 1) / per;
     const long long a_gr = g.a_group_rows > 0 ? g.a_group_rows : g.n;
-    const int tt = g.m_tok <= 8 ? 8 : 16;
+    const int per = g.a2 ? 16 : kRows, n_slices = (g.n + per - 1) / per, tt = g.m_tok <= 8 ? 8 : 16;
+    // A wave of tiles, one per SM, takes as long as about ten CTAs per SM of the warp-per-rows form (SwiGLU: eleven).
+    // Measured, warp-per-rows / tiles (us): K 256, 4096 rows x 256 (13 CTAs per SM, one wave) 57 / 27; K 1024, SwiGLU, 192
+    // rows x 4096 (20, two) 182 / 207, 512 rows (54, four) 451 / 410; K 2048, 512 rows x 3072 (20, two) 370 / 286.
+    const int n_tiles = (g.n + 127) / 128, tok = g.a2 ? 32 : 64;
+    const long long tiles = (long long)n_tiles * g.groups * ((g.m_tok + tok - 1) / tok);
+    const long long waves = (tiles + c->num_sms - 1) / c->num_sms;
+    if ((long long)n_slices * g.groups * ((g.m_tok + tt - 1) / tt) > (g.a2 ? 11 : 10) * waves * c->num_sms)
+        return launch_kernel(c->pdl, g.a2 ? gemm_simt_tiled_kernel<T, true> : gemm_simt_tiled_kernel<T, false>,
+                             dim3(n_tiles * g.groups, (g.m_tok + tok - 1) / tok), dim3(kSimtThreads), 0, s,
+                             (const T*)g.a, (const T*)g.a2, (const T*)g.b, g.n, g.k, g.m_tok, a_gr, g.b_group_rows,
+                             g.b_shared, g.b_kgroup, n_tiles, g.ep);
     return launch_kernel(c->pdl, tt == 8 ? gemm_simt_kernel<T, 8> : gemm_simt_kernel<T, 16>,
                          dim3(n_slices * g.groups, (g.m_tok + tt - 1) / tt), dim3(kSimtThreads), 0, s,
                          (const T*)g.a, (const T*)g.a2, (const T*)g.b, g.n, g.k, g.m_tok, a_gr, g.b_group_rows,

@@ -2,6 +2,8 @@
 
 The checks and tolerances are those of tests/harness.py (fp32 storage: 1e-5 element by element with the
 floor at the tensor's rms; bf16 storage: 2e-2, see there)."""
+import dataclasses
+
 import numpy as np
 import pytest
 
@@ -64,6 +66,32 @@ def test_simt_gemm_on_bf16_matches_oracle():
     """The CUDA-core GEMM on bf16 weights (a cross-check of the tensor-core GEMM)."""
     from paper_2606_02091_gb300 import FLAG_SIMT_GEMM
     _step_matches_oracle(synth.Workload("simt_bf16", _shape(d=320, ffn=192, vocab=333, block=9), (40, 3), 0.8, 35), FLAG_SIMT_GEMM)
+
+
+# the CUDA-core GEMM's 128 x 64 tiles (more than 1520 CTAs of the other form): 2048 block rows through every
+# projection, features that end inside a tile (448, 461 and 2 x 320 of 128), a fill of 4602 rows
+TILED = _shape(dtype="f32", d=448, n_draft_layers=1, ffn=320, vocab=461, block=32)
+TILED_BLOCK = synth.Workload("tiled_block", TILED, tuple(1 + b % 5 for b in range(64)), 0.8, 38, False)
+TILED_FILL = synth.Workload("tiled_fill", _shape(dtype="f32", n_draft_layers=2, head_dim=128, n_target_layers=3), (2301, 3), 0.8, 39, False)
+
+
+def test_fp32_tiles_of_many_block_rows_match_oracle():
+    _step_matches_oracle(TILED_BLOCK)
+
+
+def test_simt_tiles_of_many_block_rows_on_bf16_match_oracle():
+    from paper_2606_02091_gb300 import FLAG_SIMT_GEMM
+    w = TILED_BLOCK.with_(shape=dataclasses.replace(TILED, dtype="bf16"))
+    _step_matches_oracle(w, FLAG_SIMT_GEMM)
+
+
+@pytest.mark.parametrize("flag,kw", [("", {}), ("FLAG_FUSION_FC", dict(fusion_fc=True)), ("FLAG_DFLASH_FC", dict(dflash_fc=True)),
+                                     ("FLAG_SHARED_KV", dict(shared_kv=True))], ids=lambda x: x if isinstance(x, str) else "")
+def test_fp32_tiles_of_a_fill_match_oracle(flag, kw):
+    """The context projection (rotary epilogue, grouped weights), biased and grouped stores, a contraction across
+    stacked token groups."""
+    import paper_2606_02091_gb300 as P
+    _step_matches_oracle(TILED_FILL, getattr(P, flag) if flag else 0, **kw)
 
 
 # bf16 projections of more than 128 token rows (two-SM tiles of 256 rows x 64 to 256 features): one row
