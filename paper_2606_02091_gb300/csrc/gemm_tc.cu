@@ -691,12 +691,20 @@ cudaError_t launch_gemm_tc(dflare_ctx* c, const GemmDesc& g, cudaStream_t s, std
     const bool swiglu_tma = g.ep.kind == EPI_SWIGLU && (reinterpret_cast<uintptr_t>(g.ep.out) & 15u) == 0 && g.ep.ldo % 8 == 0;
     const bool f32_tma = g.ep.kind == EPI_F32 && !a.pair && (reinterpret_cast<uintptr_t>(g.ep.out) & 15u) == 0 && g.ep.ldo % 4 == 0;
     if (swiglu_tma || f32_tma) {
-        // (every tile counts four rows more for its hand-overs: near-ties go to the taller tile. 233484 entries, d 2560: 17
-        // waves of 96 rows against 25 of 64, 60 tokens 195.4 / 239.6 us, 15 tokens 180.3 / 180.5)
+        // A gate/up tile counts four rows more for its hand-overs. A logit tile of bn tokens counts bn^2 / 160 more, and
+        // 64 rows are taken only where one wave holds them all: at few tokens its weights' stream covers the rest, at
+        // many the tokens' own stream and the multiplication of 128 rows do not shrink with it. Measured (d 4096, us of
+        // tiles of 128 / 96 / 64 rows): 65024 entries (4 / 5 / 7 waves) 30 tokens 84.5 / 80.6 / 82.5, 60 tokens
+        // 86.7 / 88.9 / 107.6, 105 tokens 95.1 / 101.5 / 125.9; 128256 (7 / 9 / 14) 30 tokens 157.7 / 151.0 / 161.7, 60
+        // 158.2 / 161.2 / 212.8, 105 174.4 / 185.6 / 247.5; 100352 (6 / 7 / 11) 60 131.5 / 126.5 / 167.7. Over ten
+        // vocabularies, three widths and 15 to 105 tokens the choice is 4 % behind the best of the three at most, but for
+        // 65024 entries at d 2048 and 60 tokens (8 %).
         long long best_cost = 0;
         for (int bm = kBM; bm >= 64; bm -= swiglu_tma ? 16 : 32) {
             const long long t = (long long)g.groups * ((g.n + bm - 1) / bm) * a.tok_tiles;
-            const long long cost = (t + c->num_sms - 1) / c->num_sms * (bm + 4);
+            const long long waves = (t + c->num_sms - 1) / c->num_sms;
+            if (!swiglu_tma && bm == 64 && waves > 1) continue;
+            const long long cost = waves * (160 * bm + (swiglu_tma ? 160 * 4 : a.bn * a.bn));
             if (bm == kBM || cost < best_cost) {
                 best_cost = cost;
                 a.bm = bm;
