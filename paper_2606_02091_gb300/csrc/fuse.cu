@@ -591,21 +591,26 @@ cudaError_t fuse_layers_t(dflare_ctx* c, const void* hidden, int n_max, void* fu
     T* Fo = static_cast<T*>(fused_out);
     // Context fill: CTAs of d / 8 threads, or of d / 16 where six to eight draft layers take two feature groups per
     // thread, two per SM when their registers allow (rings of about 100 KB), else one (about 200 KB); at most kMaxNS
-    // stages. A producer warp refills the ring up to 1024 features, or 2048 at six to eight draft layers (where its
-    // CTA has registers for one group's sums), and for up to kFewRows target rows. Across those lines, 2048 positions,
-    // by turns / producer warp (us): d 1024 D 4 T 36 45.2 / 42.9, d 1536 D 2 T 24
-    // 10 % behind with the producer warp, d 2048 D 4 T 8 33.6 / 31.6, d 2048 D 6 T 36 121.7 / 102.4, fp32 d 1024 D 2
-    // T 12 31.6 / 31.6.
+    // stages. A producer warp refills the ring up to 1024 features, or 2560 at six to eight draft layers (where its
+    // CTA has registers for one group's sums), and for up to kFewRows target rows, unless two CTAs fit on an SM only
+    // without it. Across those lines, 2048 positions, by turns / producer warp (us): d 1024 D 4 T 36 45.2 / 42.9, d 1536
+    // D 2 T 24 10 % behind with the producer warp, d 2048 D 4 T 8 33.6 / 31.6, d 2048 D 6 T 36 121.7 / 102.4, fp32 d 1024
+    // D 2 T 12 31.6 / 31.6; d 2560 D 8 T 36 1.19 times by turns. (Six to eight draft layers of more features
+    // stay by turns: the producer's CTA would spill.)
     const int Dn = g.n_draft_layers, nf = Dn <= 5 ? 1 : 2, d_threads = (g.d / 8 + 31) / 32 * 32;   // (d <= 4096)
-    const bool prod = Dn > 5 ? g.d <= 2048 : g.d <= 1024 || (g.n_target_layers <= kFewRows<T> && (Dn < 5 || g.d <= 2048));
-    const size_t stage_bytes = (size_t)(prod ? kRowsPerStage<T, true> : kRowsPerStage<T, false>) * g.d * sizeof(T);
+    const size_t prod_stage = (size_t)kRowsPerStage<T, true> * g.d * sizeof(T);
+    const bool two_prod = d_threads <= (Dn <= 2 ? 320 : 256) && kMinNS * prod_stage <= kRingBytes / 2;
+    const bool few = g.n_target_layers <= kFewRows<T> && (two_prod || (Dn < 5 && d_threads > 320));
+    const bool prod = Dn > 5 ? d_threads <= 320 : g.d <= 1024 || few;
+    const size_t stage_bytes = prod ? prod_stage : (size_t)kRowsPerStage<T, false> * g.d * sizeof(T);
     if ((long long)c->batch * n_max >= 2LL * c->num_sms && Dn <= 8 && g.n_target_layers <= 64 &&
         kMinNS * stage_bytes <= kRingBytes) {
         static PerDeviceOnce rconf;
         const cudaError_t re = rconf([] {
             for (auto k : {fuse_rows_kernel<T, 4, 1>, fuse_rows_kernel<T, 5, 1>, fuse_rows_kernel<T, 8, 2>,
                            fuse_rows2_kernel<T, 4>, fuse_rows2_kernel<T, 5>, fuse_rows_prod_kernel<T, 4, 512, 1>,
-                           fuse_rows_prod_kernel<T, 5, 256, 2>, fuse_rows_prod_kernel<T, 8, 256, 1>}) {
+                           fuse_rows_prod_kernel<T, 2, 320, 2>, fuse_rows_prod_kernel<T, 5, 256, 2>,
+                           fuse_rows_prod_kernel<T, 8, 320, 1>}) {
                 cudaError_t e = cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kRingBytes);
                 if (e != cudaSuccess) return e;
             }
@@ -614,13 +619,15 @@ cudaError_t fuse_layers_t(dflare_ctx* c, const void* hidden, int n_max, void* fu
         if (re != cudaSuccess) return re;
         int ns = (int)std::min<size_t>(kMaxNS, kRingBytes / stage_bytes), per_sm = 1;
         const int ns2 = (int)std::min<size_t>(kMaxNS, kRingBytes / 2 / stage_bytes);
-        auto rk = prod ? (Dn > 5 ? fuse_rows_prod_kernel<T, 8, 256, 1>
-                          : d_threads <= 256 ? fuse_rows_prod_kernel<T, 5, 256, 2> : fuse_rows_prod_kernel<T, 4, 512, 1>)
+        auto rk = prod ? (Dn > 5 ? fuse_rows_prod_kernel<T, 8, 320, 1>
+                          : d_threads <= 256 ? fuse_rows_prod_kernel<T, 5, 256, 2>
+                          : d_threads <= 320 ? fuse_rows_prod_kernel<T, 2, 320, 2> : fuse_rows_prod_kernel<T, 4, 512, 1>)
                   : Dn <= 4 ? fuse_rows_kernel<T, 4, 1> : Dn == 5 ? fuse_rows_kernel<T, 5, 1> : fuse_rows_kernel<T, 8, 2>;
-        auto rk2 = prod ? fuse_rows_prod_kernel<T, 5, 256, 2> : Dn <= 4 ? fuse_rows2_kernel<T, 4> : fuse_rows2_kernel<T, 5>;
+        auto rk2 = prod ? (d_threads <= 256 ? fuse_rows_prod_kernel<T, 5, 256, 2> : fuse_rows_prod_kernel<T, 2, 320, 2>)
+                   : Dn <= 4 ? fuse_rows2_kernel<T, 4> : fuse_rows2_kernel<T, 5>;
         const int threads = prod ? d_threads + 32 : std::min(512 / nf, d_threads);
         int fit = 0;
-        if (Dn <= 5 && ns2 >= kMinNS && d_threads <= (prod ? 256 : 320) &&
+        if (Dn <= 5 && ns2 >= kMinNS && d_threads <= 320 &&
             cudaOccupancyMaxActiveBlocksPerMultiprocessor(&fit, rk2, threads, (size_t)ns2 * stage_bytes) ==
                 cudaSuccess && fit >= 2) {
             rk = rk2;

@@ -196,6 +196,11 @@ FILL_CASES = [
     synth.Workload("fill_d1024_D1_T1", _shape(d=1024, n_draft_layers=1, n_target_layers=1, ffn=64, block=2), (700,), 0.8, 59),
     synth.Workload("fill_d64_D5_T36", _shape(d=64, n_draft_layers=5, n_target_layers=36, ffn=64, block=2), (160, 3, 150), 0.8, 60),
     synth.Workload("fill_d2048_D5_T8", _shape(d=2048, n_draft_layers=5, n_target_layers=8, ffn=64, block=2), (305,), 0.8, 74),
+    synth.Workload("fill_d2560_D1_T1", _shape(d=2560, n_draft_layers=1, n_target_layers=1, ffn=64, block=2), (400,), 0.8, 80),
+    synth.Workload("fill_d2560_D8_T7", _shape(d=2560, n_draft_layers=8, n_target_layers=7, ffn=64, block=2), (305,), 0.8, 81),
+    synth.Workload("fill_d2304_D4_T8", _shape(d=2304, n_draft_layers=4, n_target_layers=8, ffn=64, block=2), (305,), 0.8, 82),
+    synth.Workload("fill_f32_d2560_D1_T2", _shape(dtype="f32", d=2560, n_draft_layers=1, n_target_layers=2, ffn=64, block=2), (305,), 0.8, 83),
+    synth.Workload("fill_f32_d2688_D6_T4", _shape(dtype="f32", d=2688, n_draft_layers=6, n_target_layers=4, ffn=64, block=2), (305,), 0.8, 84),
     synth.Workload("fill_d4096_D4_T8", _shape(d=4096, n_draft_layers=4, n_target_layers=8, ffn=64, block=2), (305,), 0.8, 75),
     synth.Workload("fill_f32_d2112_D6_T7", _shape(dtype="f32", d=2112, n_draft_layers=6, n_target_layers=7, ffn=64, block=2), (170, 140), 0.8, 76),
     synth.Workload("fill_f32_d1088_D2_T5", _shape(dtype="f32", d=1088, n_draft_layers=2, n_target_layers=5, ffn=64, block=2), (305,), 0.8, 77),
