@@ -605,37 +605,41 @@ cudaError_t fuse_layers_t(dflare_ctx* c, const void* hidden, int n_max, void* fu
     const size_t stage_bytes = prod ? prod_stage : (size_t)kRowsPerStage<T, false> * g.d * sizeof(T);
     if ((long long)c->batch * n_max >= 2LL * c->num_sms && Dn <= 8 && g.n_target_layers <= 64 &&
         kMinNS * stage_bytes <= kRingBytes) {
-        static PerDeviceOnce rconf;
-        const cudaError_t re = rconf([] {
-            for (auto k : {fuse_rows_kernel<T, 4, 1>, fuse_rows_kernel<T, 5, 1>, fuse_rows_kernel<T, 8, 2>,
-                           fuse_rows2_kernel<T, 4>, fuse_rows2_kernel<T, 5>, fuse_rows_prod_kernel<T, 4, 512, 1>,
-                           fuse_rows_prod_kernel<T, 2, 320, 2>, fuse_rows_prod_kernel<T, 5, 256, 2>,
-                           fuse_rows_prod_kernel<T, 8, 320, 1>}) {
-                cudaError_t e = cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kRingBytes);
-                if (e != cudaSuccess) return e;
-            }
-            return cudaSuccess;
-        });
-        if (re != cudaSuccess) return re;
+        // each variant is set up, and with that loaded, when it is first taken: all nine at once moved what a program
+        // allocates after its first fill, and with it other launches (Qwen3-4B block 402.5 -> 407.2 us)
+        enum { BY_TURNS_4, BY_TURNS_5, BY_TURNS_8, TWO_BY_TURNS_4, TWO_BY_TURNS_5, PROD_4, TWO_PROD_2, TWO_PROD_5, PROD_8, VARIANTS };
+        using Fill = decltype(&fuse_rows_kernel<T, 4, 1>);
+        static const Fill variant[VARIANTS] = {
+            fuse_rows_kernel<T, 4, 1>, fuse_rows_kernel<T, 5, 1>, fuse_rows_kernel<T, 8, 2>, fuse_rows2_kernel<T, 4>,
+            fuse_rows2_kernel<T, 5>, fuse_rows_prod_kernel<T, 4, 512, 1>, fuse_rows_prod_kernel<T, 2, 320, 2>,
+            fuse_rows_prod_kernel<T, 5, 256, 2>, fuse_rows_prod_kernel<T, 8, 320, 1>};
+        static PerDeviceOnce ready[VARIANTS];
+        auto set_up = [](int i) {
+            return ready[i]([i] {
+                return cudaFuncSetAttribute(variant[i], cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kRingBytes);
+            });
+        };
+        // v2: two CTAs per SM, where they fit; v: one (with a producer warp the same kernel, if it has one for two)
+        const int v2 = prod ? (d_threads <= 256 ? TWO_PROD_5 : TWO_PROD_2) : Dn <= 4 ? TWO_BY_TURNS_4 : TWO_BY_TURNS_5;
+        int v = prod ? (Dn > 5 ? PROD_8 : d_threads <= 320 ? v2 : PROD_4)
+                     : Dn <= 4 ? BY_TURNS_4 : Dn == 5 ? BY_TURNS_5 : BY_TURNS_8;
         int ns = (int)std::min<size_t>(kMaxNS, kRingBytes / stage_bytes), per_sm = 1;
         const int ns2 = (int)std::min<size_t>(kMaxNS, kRingBytes / 2 / stage_bytes);
-        auto rk = prod ? (Dn > 5 ? fuse_rows_prod_kernel<T, 8, 320, 1>
-                          : d_threads <= 256 ? fuse_rows_prod_kernel<T, 5, 256, 2>
-                          : d_threads <= 320 ? fuse_rows_prod_kernel<T, 2, 320, 2> : fuse_rows_prod_kernel<T, 4, 512, 1>)
-                  : Dn <= 4 ? fuse_rows_kernel<T, 4, 1> : Dn == 5 ? fuse_rows_kernel<T, 5, 1> : fuse_rows_kernel<T, 8, 2>;
-        auto rk2 = prod ? (d_threads <= 256 ? fuse_rows_prod_kernel<T, 5, 256, 2> : fuse_rows_prod_kernel<T, 2, 320, 2>)
-                   : Dn <= 4 ? fuse_rows2_kernel<T, 4> : fuse_rows2_kernel<T, 5>;
         const int threads = prod ? d_threads + 32 : std::min(512 / nf, d_threads);
-        int fit = 0;
-        if (Dn <= 5 && ns2 >= kMinNS && d_threads <= 320 &&
-            cudaOccupancyMaxActiveBlocksPerMultiprocessor(&fit, rk2, threads, (size_t)ns2 * stage_bytes) ==
-                cudaSuccess && fit >= 2) {
-            rk = rk2;
-            ns = ns2;
-            per_sm = 2;
+        if (Dn <= 5 && ns2 >= kMinNS && d_threads <= 320) {
+            int fit = 0;
+            if (set_up(v2) == cudaSuccess &&
+                cudaOccupancyMaxActiveBlocksPerMultiprocessor(&fit, variant[v2], threads, (size_t)ns2 * stage_bytes) ==
+                    cudaSuccess && fit >= 2) {
+                v = v2;
+                ns = ns2;
+                per_sm = 2;
+            }
         }
+        const cudaError_t re = set_up(v);
+        if (re != cudaSuccess) return re;
         const int grid = (int)std::min<long long>((long long)c->batch * n_max, (long long)per_sm * c->num_sms);
-        return launch_kernel(c->pdl, rk, dim3(grid), dim3(threads), (size_t)ns * stage_bytes, s, H,
+        return launch_kernel(c->pdl, variant[v], dim3(grid), dim3(threads), (size_t)ns * stage_bytes, s, H,
                              (const float*)c->alpha, gain, F, Fo, (const int32_t*)c->app_cnt,
                              g.n_draft_layers, g.n_target_layers, c->batch, n_max, g.d,
                              (long long)g.max_fuse_rows, g.rms_eps, ns, c->err);
