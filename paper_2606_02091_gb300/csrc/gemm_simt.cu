@@ -15,6 +15,8 @@
 // drafter (d 256, 4 layers, block 8) went from 968 to 158 us, and to 134 with two chunks of K per round.
 #include "epilogue.cuh"
 
+#include <algorithm>
+
 namespace dfl {
 namespace {
 
@@ -135,26 +137,28 @@ __global__ void __launch_bounds__(kSimtThreads) gemm_simt_kernel(
     }
 }
 
-// Many token rows: one CTA computes 128 weight rows x 64 tokens (SwiGLU: 128 of gate, the same 128 of up x 32
-// tokens), 8 x 4 sums (2 x 8 x 2) per thread, K in chunks of 16 through two shared-memory buffers, the next
-// chunk's loads in flight behind the FMAs. The warp-per-rows form, whose eight warps each load the tokens for
-// themselves, had fallen behind the one before it here: fp32 (us, the one before / warp per rows / tiles), 16384 rows
-// x 512 x 1024 1180 / 1389 / 508, 32768 x 512 x 512 1175 / 1538 / 532, 8192 x 256 x 256 96 / 105 / 47. Bound by the
-// FMAs and the shared-memory reads that feed them.
-// A thread adds a chunk's products in two chains of 8, four chunks' sums to a partial sum and that to the total:
-// the error against 64 bits is that of the warp-per-rows form at K 256 (8.1e-8 of the result's rms) and below it
-// beyond (K 2048 1.2e-7 / 1.6e-7; chains of 64 would have 1.5e-7 at K 256).
-constexpr int kTileK = 16, kFlush = 4;
-template <class T, bool DUAL>
-__global__ void __launch_bounds__(kSimtThreads) gemm_simt_tiled_kernel(
+// Many token rows, or a short K under many weight rows: one CTA computes 128 weight rows x TOK tokens (SwiGLU: 128 of
+// gate, the same 128 of up x 32 tokens), TOK 64 as 8 x 4 sums per thread (2 x 8 x 2), TOK 16 as 8 x 1, K in chunks of
+// 16 through two shared-memory buffers, the next chunk's loads in flight behind the FMAs. Bound by the FMAs and the
+// shared-memory reads that feed them. The warp-per-rows form, whose eight warps each load the tokens for themselves
+// and pay its butterfly and its rounds of 128 k whatever K is, had fallen behind the one before it here (us, the one
+// before / warp per rows / tiles): K 1024, 16384 rows x 512 1180 / 1389 / 508; K 512, 32768 x 512 1174 / 1522 / 535; K 256,
+// 8192 x 256 97 / 106 / 47; K 64, 151936 features, 15 rows 31 / 65 / 33 (TOK 16), 60 rows 98 / 246 / 61; K 192, 151936
+// features, 15 rows 84 / 105 / 82. What is left behind: 151936 features at K 64 and 128, up to 30 rows, 4 to 15 %.
+// A thread adds a chunk's products in four chains of 4, which are added pairwise. TREE: chunks are added pairwise too,
+// and each four of them to the total (K up to 128, at 20 % more time than without); otherwise four in a row and that to the
+// total. The error against 64 bits is then no larger than the warp-per-rows form's (rms, of the result's, in 1e-8;
+// warp per rows / tree / no tree): K 64 6.77 / 6.77 / 6.90, K 128 7.29 / 7.29 / 7.41, K 192 7.85 / - / 7.74, K 256
+// 8.14 / - / 8.01, K 2048 15.7 / - / 12.7. (Chains of 8 would save 5 % and have 7.77 at K 128 and 8.33 at K 256.)
+constexpr int kTileK = 16, kChain = 4;
+template <class T, bool DUAL, int TOK, bool TREE>
+__global__ void __launch_bounds__(kSimtThreads, TOK == 16 ? 2 : 1) gemm_simt_tiled_kernel(
     const T* __restrict__ A, const T* __restrict__ A2, const T* __restrict__ Bm, int n, int k, int m_tok,
     long long a_group_rows, long long b_group_rows, int b_shared, int b_kgroup, int n_tiles, EpiParams ep) {
-    constexpr int NA = DUAL ? 2 : 1, TOK = 64 / NA, TPT = TOK / 16;   // tokens per CTA and thread
+    constexpr int NA = DUAL ? 2 : 1, TPT = TOK / 16;   // accumulators, tokens per thread
     constexpr int LDA = 128 + 4, LDB = TOK + 4;
     constexpr int OPS = 2 * kTileK * (NA * LDA + LDB), TILES = NA * TOK * 128;
     __shared__ __align__(16) float buf[OPS > TILES ? OPS : TILES];   // operands, then the epilogue's tiles
-    pdl_wait();
-    pdl_trigger();   // after the wait: see gemm_tc_kernel
     const int n_tile = blockIdx.x % n_tiles, group = blockIdx.x / n_tiles, tok0 = blockIdx.y * TOK;
     const int tid = threadIdx.x, tx = tid & 15, ty = tid >> 4;
     const T* Bg = Bm + (size_t)(b_shared || b_kgroup > 0 ? 0 : group) * b_group_rows * k;
@@ -176,11 +180,13 @@ __global__ void __launch_bounds__(kSimtThreads) gemm_simt_tiled_kernel(
     auto As = [&](int st, int a) { return buf + (st * NA + a) * kTileK * LDA; };
     auto Bs = [&](int st) { return buf + 2 * NA * kTileK * LDA + st * kTileK * LDB; };
     float4 ra[NA][2], rb = make_float4(0.f, 0.f, 0.f, 0.f);
-    auto load = [&](int k0) {
+    auto load_a = [&](int k0) {
 #pragma unroll
         for (int a = 0; a < NA; ++a)
 #pragma unroll
             for (int h = 0; h < 2; ++h) ra[a][h] = ld4(ap[a][h] + k0);
+    };
+    auto load_b = [&](int k0) {
         if (lb) rb = ld4(b_at(k0));
     };
     auto put = [&](float* d, int ld, float4 v) {
@@ -197,23 +203,30 @@ __global__ void __launch_bounds__(kSimtThreads) gemm_simt_tiled_kernel(
         if (lb) put(Bs(st) + lk * LDB + lr, LDB, rb);
     };
     constexpr int S = NA * 8 * TPT;                 // sums of a thread, [accumulator][feature][token]
-    float acc[S], part[S];
+    float acc[S], part[S], pair[S];
 #pragma unroll
     for (int i = 0; i < S; ++i) acc[i] = part[i] = 0.f;
-    load(0);
+    load_a(0);
+    pdl_wait();
+    pdl_trigger();   // after the wait: see gemm_tc_kernel
+    load_b(0);
     store(0);
     __syncthreads();
     const int chunks = k / kTileK;   // (k is a multiple of 64)
     for (int c = 0; c < chunks; ++c) {
         const int st = c & 1;
-        if (c + 1 < chunks) load((c + 1) * kTileK);
-        float sum[2][S];
+        if (c + 1 < chunks) {
+            load_a((c + 1) * kTileK);
+            load_b((c + 1) * kTileK);
+        }
+        constexpr int NC = kTileK / kChain;
+        float sum[NC][S];
 #pragma unroll
-        for (int h = 0; h < 2; ++h) {
+        for (int h = 0; h < NC; ++h) {
 #pragma unroll
             for (int i = 0; i < S; ++i) sum[h][i] = 0.f;
 #pragma unroll
-            for (int kk = h * 8; kk < h * 8 + 8; ++kk) {
+            for (int kk = h * kChain; kk < (h + 1) * kChain; ++kk) {
                 float b[TPT];
 #pragma unroll
                 for (int t = 0; t < TPT; ++t) b[t] = Bs(st)[kk * LDB + ty * TPT + t];
@@ -233,12 +246,31 @@ __global__ void __launch_bounds__(kSimtThreads) gemm_simt_tiled_kernel(
             }
         }
 #pragma unroll
-        for (int i = 0; i < S; ++i) part[i] += sum[0][i] + sum[1][i];
-        if (c % kFlush == kFlush - 1) {
+        for (int i = 0; i < S; ++i) sum[0][i] = (sum[0][i] + sum[1][i]) + (sum[2][i] + sum[3][i]);
+        if (TREE) {
+            if (!(c & 1)) {
 #pragma unroll
-            for (int i = 0; i < S; ++i) {
-                acc[i] += part[i];
-                part[i] = 0.f;
+                for (int i = 0; i < S; ++i) pair[i] = sum[0][i];
+            } else {
+#pragma unroll
+                for (int i = 0; i < S; ++i) pair[i] += sum[0][i];
+                if (!(c & 2)) {
+#pragma unroll
+                    for (int i = 0; i < S; ++i) part[i] = pair[i];
+                } else {
+#pragma unroll
+                    for (int i = 0; i < S; ++i) acc[i] += part[i] + pair[i];
+                }
+            }
+        } else {
+#pragma unroll
+            for (int i = 0; i < S; ++i) part[i] += sum[0][i];
+            if ((c & 3) == 3) {
+#pragma unroll
+                for (int i = 0; i < S; ++i) {
+                    acc[i] += part[i];
+                    part[i] = 0.f;
+                }
             }
         }
         if (c + 1 < chunks) store(st ^ 1);   // (read two chunks ago, before the last barrier)
@@ -264,17 +296,30 @@ template <class T>
 cudaError_t launch_t(dflare_ctx* c, const GemmDesc& g, cudaStream_t s) {
     const long long a_gr = g.a_group_rows > 0 ? g.a_group_rows : g.n;
     const int per = g.a2 ? 16 : kRows, n_slices = (g.n + per - 1) / per, tt = g.m_tok <= 8 ? 8 : 16;
-    // A wave of tiles, one per SM, takes as long as about ten CTAs per SM of the warp-per-rows form (SwiGLU: eleven).
-    // Measured, warp-per-rows / tiles (us): K 256, 4096 rows x 256 (13 CTAs per SM, one wave) 57 / 27; K 1024, SwiGLU, 192
-    // rows x 4096 (20, two) 182 / 207, 512 rows (54, four) 451 / 410; K 2048, 512 rows x 3072 (20, two) 370 / 286.
-    const int n_tiles = (g.n + 127) / 128, tok = g.a2 ? 32 : 64;
-    const long long tiles = (long long)n_tiles * g.groups * ((g.m_tok + tok - 1) / tok);
-    const long long waves = (tiles + c->num_sms - 1) / c->num_sms;
-    if ((long long)n_slices * g.groups * ((g.m_tok + tt - 1) / tt) > (g.a2 ? 11 : 10) * waves * c->num_sms)
-        return launch_kernel(c->pdl, g.a2 ? gemm_simt_tiled_kernel<T, true> : gemm_simt_tiled_kernel<T, false>,
-                             dim3(n_tiles * g.groups, (g.m_tok + tok - 1) / tok), dim3(kSimtThreads), 0, s,
+    const long long warp_ctas = (long long)n_slices * g.groups * ((g.m_tok + tt - 1) / tt);
+    const int n_tiles = (g.n + 127) / 128;
+    auto tiled = [&](auto kernel, int tok) {
+        return launch_kernel(c->pdl, kernel, dim3(n_tiles * g.groups, (g.m_tok + tok - 1) / tok), dim3(kSimtThreads), 0, s,
                              (const T*)g.a, (const T*)g.a2, (const T*)g.b, g.n, g.k, g.m_tok, a_gr, g.b_group_rows,
                              g.b_shared, g.b_kgroup, n_tiles, g.ep);
+    };
+    // A wave of tiles, one per SM, takes as long as about ten CTAs per SM of the warp-per-rows form (SwiGLU: eleven), and
+    // as six where K is short, which that form pays by 128 (SwiGLU at K 64: four). Measured, warp-per-rows / tiles (us):
+    // K 64, 120 rows x 8192 (13 CTAs per SM, one wave) 33 / 12; K 256, 4096 x 256 (13, one) 57 / 27; K 1024, SwiGLU, 192 x 4096
+    // (20, two) 182 / 207, 512 (54, four) 451 / 404; K 2048, 512 x 3072 (20, two) 370 / 288.
+    const int tok = g.a2 ? 32 : 64, limit = g.a2 && g.k <= 64 ? 4 : g.k <= 192 ? 6 : g.a2 ? 11 : 10;
+    const long long sms = c->num_sms, tiles = (long long)n_tiles * g.groups * ((g.m_tok + tok - 1) / tok);
+    if (warp_ctas > limit * ((tiles + sms - 1) / sms) * sms) {
+        if (g.k <= 128) return tiled(g.a2 ? gemm_simt_tiled_kernel<T, true, 32, true> : gemm_simt_tiled_kernel<T, false, 64, true>, tok);
+        return tiled(g.a2 ? gemm_simt_tiled_kernel<T, true, 32, false> : gemm_simt_tiled_kernel<T, false, 64, false>, tok);
+    }
+    // Few token rows under many weight rows at a short K: tiles of 16 tokens, from three CTAs per SM of the warp-per-rows
+    // form at K 64 and twelve at 128 and 192 (above 8 tokens there), and where 128 rows are mostly not padding.
+    // Measured, warp-per-rows / these: K 64, 30 rows x 8192 (3.4 CTAs per SM) 12.2 / 10.1, 15 x 32000 (6.6) 18.4 / 12.2; K 128,
+    // 7 x 32000 (6.6) 16.4 / 18.4, 7 x 151936 (31) 59 / 55; K 192, 7 x 151936 65 / 80, 15 rows 105 / 82.
+    const long long tiles16 = (long long)n_tiles * g.groups * ((g.m_tok + 15) / 16);
+    if (!g.a2 && g.k <= 192 && (g.k <= 128 || g.m_tok > 8) && warp_ctas > 3 * std::max(tiles16, (g.k <= 64 ? 1 : 4) * sms))
+        return tiled(gemm_simt_tiled_kernel<T, false, 16, true>, 16);
     return launch_kernel(c->pdl, tt == 8 ? gemm_simt_kernel<T, 8> : gemm_simt_kernel<T, 16>,
                          dim3(n_slices * g.groups, (g.m_tok + tt - 1) / tt), dim3(kSimtThreads), 0, s,
                          (const T*)g.a, (const T*)g.a2, (const T*)g.b, g.n, g.k, g.m_tok, a_gr, g.b_group_rows,

@@ -85,6 +85,30 @@ def test_simt_tiles_of_many_block_rows_on_bf16_match_oracle():
     _step_matches_oracle(w, FLAG_SIMT_GEMM)
 
 
+# the tiles of a short K: 16 tokens in the LM head (240 rows x 1003; 15 x 58401 at K 192) and in Q/K/V (256 x 1024, rotary), more
+# in gate/up (256 x 640) and, with 16 query heads and 2049 features, in Q/K/V and the LM head
+SHORT_K = [
+    synth.Workload("short_64", _shape(dtype="f32", d=64, n_draft_layers=1, n_q_heads=8, n_kv_heads=4, ffn=640, vocab=1003,
+                                      block=16), tuple(1 + b % 5 for b in range(16)), 0.8, 60, False),
+    synth.Workload("short_64_wide", _shape(dtype="f32", d=64, n_draft_layers=1, n_q_heads=16, n_kv_heads=8, ffn=64, vocab=2049,
+                                           block=16), tuple(1 + b % 5 for b in range(16)), 0.8, 61, False),
+    synth.Workload("short_128", _shape(dtype="f32", d=128, n_draft_layers=1, n_q_heads=16, n_kv_heads=8, ffn=64, vocab=2049,
+                                       block=16), tuple(1 + b % 5 for b in range(16)), 0.8, 62, False),
+    synth.Workload("short_192", _shape(dtype="f32", d=192, n_draft_layers=1, vocab=58401, block=16), (3,), 0.8, 63, False),
+]
+
+
+@pytest.mark.parametrize("w", SHORT_K, ids=lambda w: w.name)
+def test_fp32_tiles_of_a_short_k_match_oracle(w):
+    _step_matches_oracle(w)
+
+
+def test_simt_tiles_of_a_short_k_on_bf16_match_oracle():
+    from paper_2606_02091_gb300 import FLAG_SIMT_GEMM
+    w = SHORT_K[0]
+    _step_matches_oracle(w.with_(shape=dataclasses.replace(w.shape, dtype="bf16")), FLAG_SIMT_GEMM)
+
+
 @pytest.mark.parametrize("flag,kw", [("", {}), ("FLAG_FUSION_FC", dict(fusion_fc=True)), ("FLAG_DFLASH_FC", dict(dflash_fc=True)),
                                      ("FLAG_SHARED_KV", dict(shared_kv=True))], ids=lambda x: x if isinstance(x, str) else "")
 def test_fp32_tiles_of_a_fill_match_oracle(flag, kw):
