@@ -7,6 +7,7 @@ import dataclasses
 import numpy as np
 import pytest
 
+import oracle as O
 import synth
 from tests.harness import GpuSide, check_kv, check_rows, check_tokens, f64, oracle_for
 
@@ -264,6 +265,25 @@ def test_copies_to_aligned_and_unaligned_buffers_agree(vocab, block, sampled):
         assert got[-1][2].any() and (block == 1 or got[-1][1].all())
     for a, b in zip(*got):
         np.testing.assert_array_equal(a, b)
+
+
+@pytest.mark.parametrize("batch,block", [(9, 2), (31, 8), (33, 17), (64, 32)])
+def test_verification_of_many_sequences_matches_oracle(batch, block):
+    """The acceptance of up to four sequences at a time per warp: every prefix length, both entry points."""
+    import torch
+    w = synth.Workload("many", _shape(block=block, vocab=301), (1,) * batch, 0.8, 64)
+    g, V, rng = GpuSide(w), w.shape.vocab, np.random.default_rng(64)
+    draft = rng.integers(0, V, (batch, block - 1)).astype(np.int32)
+    lg = rng.standard_normal((batch, block, V)).astype(np.float32)
+    for b in range(batch):
+        for k in range(b % block):
+            lg[b, k, draft[b, k]] = 20.0
+    want = [O.verify_from_logits(draft[b], lg[b]) for b in range(batch)]
+    d, t = torch.from_numpy(draft).cuda(), torch.from_numpy(lg).cuda()
+    for call, arg in ((g.lib.verify_logits, t), (g.lib.verify_accept, t.argmax(-1).int())):
+        acc, nxt = (torch.zeros(batch, dtype=torch.int32, device="cuda") for _ in range(2))
+        call(d, arg, acc, nxt)
+        assert list(zip(acc.cpu().tolist(), nxt.cpu().tolist())) == want
 
 
 def test_verification_reports_every_phase():
